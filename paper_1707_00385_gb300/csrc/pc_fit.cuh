@@ -599,7 +599,11 @@ __device__ __forceinline__ void reduce_lanes(Moments2& m) {
 // instead of one packed add per pair; the same values, so the same bits.  The
 // normal field alone takes it (GB300, 4096 x 4096: 0.430 -> 0.417 ms); the
 // fused kernel keeps the add, whose registers are all in use.
-template <int RN, bool CONST_DU = false>
+// FULL: every point of the patch is valid (the caller has checked it): no
+// masks and no count, 13 packed operations a pair instead of 14 and the two
+// selects.  With M = 1 each masked value is the same single rounding and the
+// count is exact, so the bits are those of the masked form.
+template <int RN, bool CONST_DU = false, bool FULL = false>
 __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_rt, float ap, float bp, float Zp,
                                                const Camera& cam, float det_tol, float& nx, float& ny,
                                                float& nz) {
@@ -620,14 +624,19 @@ __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_r
             const f32x2 DU = CONST_DU && RN > 0 ? pack((float)du, -(float)du) : DUi;
             const float a = za[du], b = zb[-du];
             const f32x2 Z = pack(a, b);  // 0 where invalid
-            const f32x2 M = pack(a > 0.f ? 1.f : 0.f, b > 0.f ? 1.f : 0.f);
             // masked coordinates, exactly 0 for an invalid point (Z = 0, M = 0) and
             // the unmasked values otherwise: M (Z - Zp), du Z + ap M (Z - Zp), ...;
             // M^2 = M, so the products of masked coordinates are masked too
-            const f32x2 MZ = fma2(M, NZP, Z);
+            f32x2 MZ;
+            if (FULL) {
+                MZ = add2(Z, NZP);
+            } else {
+                const f32x2 M = pack(a > 0.f ? 1.f : 0.f, b > 0.f ? 1.f : 0.f);
+                MZ = fma2(M, NZP, Z);
+                N = add2(N, M);
+            }
             const f32x2 MX = fma2(DU, Z, mul2(AP, MZ));
             const f32x2 MY = fma2(DV, Z, mul2(BP, MZ));
-            N = add2(N, M);
             SX = add2(SX, MX);
             SY = add2(SY, MY);
             SZ = add2(SZ, MZ);
@@ -639,7 +648,8 @@ __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_r
             if (!(CONST_DU && RN > 0)) DUi = add2(DUi, STEP);
         }
     }
-    const float n = hsum(N) + 1.f;  // + the centre, at x' = y' = z' = 0
+    // + the centre, at x' = y' = z' = 0
+    const float n = FULL ? (float)((2 * rn + 1) * (2 * rn + 1)) : hsum(N) + 1.f;
     const float sx = hsum(SX), sy = hsum(SY), sz = hsum(SZ);
     const float sxx = hsum(SXX), sxy = hsum(SXY), syy = hsum(SYY), sxz = hsum(SXZ), syz = hsum(SYZ);
     // centred second moments M' and v' (shift by the centre point first)

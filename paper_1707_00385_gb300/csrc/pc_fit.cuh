@@ -1,8 +1,8 @@
 // pc_fit.cuh -- the fused per-pixel curvature kernel (sm_103a).
 //
 // One CTA computes a 32 x th tile of output pixels (th = 8 or 4 with one
-// thread per pixel; th = 4, 2, 1 with lane groups of 2, 4, 8 per pixel).  The
-// CTA first stages the tile's range values plus a halo of max(r, r_n) pixels
+// thread per pixel, or a taller one 16 or 8 wide at the right edge; th = 4, 2,
+// 1 with lane groups of 2, 4, 8 per pixel).  The CTA first stages the tile's range values plus a halo of max(r, r_n) pixels
 // into shared memory as two planes, Z and c, c = 1 for a valid range and +inf
 // for none (outside the image, zero, negative or not finite), and counts the
 // valid window points of every pixel row by row.  Each thread then runs the
@@ -173,47 +173,59 @@ __device__ __forceinline__ f32x2 residual2(const Coef2& k, f32x2 X, f32x2 Y, f32
     return fma2(GA, X, fma2(GB, Y, fma2(k.nhs, Hs, k.nts)));
 }
 
-// One symmetric pair: residuals (the quadric of Sec. 3.2 in the local frame),
-// Cauchy weights, Jacobian rows and the 26 sums (the eps sums scaled by sigma).
+// What the sums take from a symmetric pair: local coordinates, Jacobian rows,
+// scaled residual and weight.
+struct PairState {
+    f32x2 X, Y, NJ0, J1, E, Wt;
+};
+
+// A symmetric pair's state: residuals (the quadric of Sec. 3.2 in the local
+// frame), Cauchy weights and Jacobian rows.
 // C = (c_a, c_b), 1 valid / +inf invalid.  thr bounds e^2 when REJECT.
-// c holds the compensations of the sums when KAHAN (unused otherwise).
 // FIRST: the first iteration, where A = B = C = 0, so that e = -sigma (h + t_z),
 // j1 = x, -j0 = y, and five sums repeat others (first_iteration_sums fills them).
-template <bool REJECT, bool KAHAN, bool FIRST>
-__device__ __forceinline__ void visit2(Moments2& m, Moments2& c, const Coef2& k, float za, float zb,
-                                       float ca, float cb, f32x2 DU, f32x2 RX, f32x2 RY, f32x2 RH,
-                                       float thr) {
-    f32x2 X, Y, Hs, GA, GB;
-    local_xyz2(k, pack(za, zb), DU, RX, RY, RH, X, Y, Hs);
-    const f32x2 E = FIRST ? fma2(k.nhs, Hs, k.nts) : residual2(k, X, Y, Hs, GA, GB);
+template <bool REJECT, bool FIRST>
+__device__ __forceinline__ PairState pair_state(const Coef2& k, float za, float zb, float ca, float cb, f32x2 DU,
+                                                f32x2 RX, f32x2 RY, f32x2 RH, float thr) {
+    PairState p;
+    f32x2 Hs, GA, GB;
+    local_xyz2(k, pack(za, zb), DU, RX, RY, RH, p.X, p.Y, Hs);
+    p.E = FIRST ? fma2(k.nhs, Hs, k.nts) : residual2(k, p.X, p.Y, Hs, GA, GB);
     float da, db;
-    unpack(fma2(E, E, pack(ca, cb)), da, db);
+    unpack(fma2(p.E, p.E, pack(ca, cb)), da, db);
     float wa = rcp_approx(da), wb = rcp_approx(db);
     if (REJECT) {
         float ea, eb;
-        unpack(mul2(E, E), ea, eb);
+        unpack(mul2(p.E, p.E), ea, eb);
         wa = ea <= thr ? wa : 0.f;
         wb = eb <= thr ? wb : 0.f;
     }
-    const f32x2 Wt = pack(wa, wb);
-    const f32x2 NJ0 = FIRST ? Y : fma2(GB, Hs, Y);
-    const f32x2 J1 = FIRST ? X : fma2(GA, Hs, X);
-    const f32x2 XX = mul2(X, X), XY = mul2(X, Y), YY = mul2(Y, Y);
-    const f32x2 WE = mul2(Wt, E), WJ0 = mul2(Wt, NJ0), WJ1 = mul2(Wt, J1);
-    const f32x2 WXX = mul2(Wt, XX), WYY = mul2(Wt, YY);
+    p.Wt = pack(wa, wb);
+    p.NJ0 = FIRST ? p.Y : fma2(GB, Hs, p.Y);
+    p.J1 = FIRST ? p.X : fma2(GA, Hs, p.X);
+    return p;
+}
+
+// The 26 sums of a pair (the eps sums scaled by sigma).  c holds the
+// compensations of the sums when KAHAN (unused otherwise).
+template <bool KAHAN, bool FIRST>
+__device__ __forceinline__ void add_pair(Moments2& m, Moments2& c, const PairState& p) {
+    const f32x2 XX = mul2(p.X, p.X), XY = mul2(p.X, p.Y), YY = mul2(p.Y, p.Y);
+    const f32x2 WE = mul2(p.Wt, p.E), WJ0 = mul2(p.Wt, p.NJ0), WJ1 = mul2(p.Wt, p.J1);
+    const f32x2 WXX = mul2(p.Wt, XX), WYY = mul2(p.Wt, YY);
     // The sums are ordered so that each multiply-add shares an operand with the
     // one before it: a packed FMA whose three operands are all fresh registers
     // issues at about 0.7 of the FP32 rate, one with a repeated operand at ~0.9.
     acc_add<KAHAN>(m.s0, c.s0, WJ0);
     acc_add<KAHAN>(m.s1, c.s1, WJ1);
-    acc_add<KAHAN>(m.sw, c.sw, Wt);
+    acc_add<KAHAN>(m.sw, c.sw, p.Wt);
     acc_add<KAHAN>(m.sxx, c.sxx, WXX);
     acc_add<KAHAN>(m.syy, c.syy, WYY);
     acc_add<KAHAN>(m.ge, c.ge, WE);
     if (!FIRST) {
         // with j1 = x, -j0 = y these are sum w y^2, w x y, w x^2, w x^2 y, w x y^2
-        acc_fma<KAHAN>(m.h00, c.h00, WJ0, NJ0);
-        acc_fma<KAHAN>(m.h01, c.h01, WJ0, J1);
+        acc_fma<KAHAN>(m.h00, c.h00, WJ0, p.NJ0);
+        acc_fma<KAHAN>(m.h01, c.h01, WJ0, p.J1);
     }
     acc_fma<KAHAN>(m.h03, c.h03, WJ0, XX);
     acc_fma<KAHAN>(m.h04, c.h04, WJ0, XY);
@@ -223,15 +235,15 @@ __device__ __forceinline__ void visit2(Moments2& m, Moments2& c, const Coef2& k,
         acc_fma<KAHAN>(m.h14, c.h14, WJ1, XY);
     }
     acc_fma<KAHAN>(m.h13, c.h13, WJ1, XX);
-    if (!FIRST) acc_fma<KAHAN>(m.h11, c.h11, WJ1, J1);
-    acc_fma<KAHAN>(m.g1, c.g1, WE, J1);
-    acc_fma<KAHAN>(m.g0, c.g0, WE, NJ0);
+    if (!FIRST) acc_fma<KAHAN>(m.h11, c.h11, WJ1, p.J1);
+    acc_fma<KAHAN>(m.g1, c.g1, WE, p.J1);
+    acc_fma<KAHAN>(m.g0, c.g0, WE, p.NJ0);
     acc_fma<KAHAN>(m.g3, c.g3, WE, XX);
     acc_fma<KAHAN>(m.g4, c.g4, WE, XY);
     acc_fma<KAHAN>(m.g5, c.g5, WE, YY);
     acc_fma<KAHAN>(m.m04, c.m04, WYY, YY);
     acc_fma<KAHAN>(m.m13, c.m13, WYY, XY);
-    acc_fma<KAHAN>(m.sxy, c.sxy, Wt, XY);
+    acc_fma<KAHAN>(m.sxy, c.sxy, p.Wt, XY);
     acc_fma<KAHAN>(m.m31, c.m31, WXX, XY);
     acc_fma<KAHAN>(m.m40, c.m40, WXX, XX);
     acc_fma<KAHAN>(m.m22, c.m22, WXX, YY);
@@ -671,18 +683,20 @@ __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_r
     return true;
 }
 
-// The whole method for one 32 x TH output tile (tile column tx_, tile row ty_)
-// of frame f.  Called by every thread of the CTA (32 x TH G threads, TH G
-// warps); contains one __syncthreads and leaves shared memory in use until it
-// returns (callers that reuse smem synchronise first).
+// The whole method for one output tile of frame f: TW x TH' pixels from (ub, vb),
+// TW = 2^lg, TH' = 32 TH / TW (32 x TH, or one of the strip shapes of Tiling),
+// cut off at row vend.  Called by every thread of the CTA (32 x TH G threads,
+// TH G warps); contains one __syncthreads and leaves shared memory in use until
+// it returns (callers that reuse smem synchronise first).
 // RW > 0: window radius RW and sampling stride RS fixed at compile time,
 // columns unrolled.  RW == 0: radius and stride from cfg.
 // G: lanes per pixel.  G = 1: one thread per pixel.  G > 1: G adjacent lanes
 // share a pixel's window rows (for_each_pair_lanes) and sum their moments
 // (reduce_lanes) before each solve, which every lane of the group repeats;
 // only the order of the moment sums differs from G = 1.
-template <int RW, bool REJECT, int PREC = 0, int TH = 8, int G = 1, int RS = 1>
-__device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cfg, int tx_, int ty_,
+// STRIPS: the tile may be a strip (Tiling), else 32 x TH.
+template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS>
+__device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cfg, int ub, int vb, int lg, int vend,
                                          float* smem) {
     constexpr bool KAHAN = (PREC & PREC_KAHAN) != 0;
     constexpr int FMT = prec_format(PREC);
@@ -702,15 +716,17 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
     const int s = RW > 0 ? RS : cfg.stride;
     const int r0 = (r / s) * s;   // largest sampled offset
     const int halo = r > cfg.rn ? r : cfg.rn;
-    const int SW = TILE_W + 2 * halo;
-    const int SH = TH + 2 * halo;
+    if (!STRIPS) lg = 5;
+    const int TW = 1 << lg;
+    const int SWU = TW + 2 * halo;                              // staged columns
+    int SW = STRIPS ? tile_pitch(TW, halo) : TILE_W + 2 * halo;  // row pitch
+    const int SH = ((TILE_W * TH) >> lg) + 2 * halo;
+    const int tid = threadIdx.y * TILE_W + threadIdx.x;
     float* tz = smem;                       // Z plane, SH x SW
     float* tcv = smem + SW * SH;            // c plane
     int* rcnt = (int*)(tcv + SW * SH);      // valid window points per (tile row, pixel column)
     // folded totals: FOLD_SUMS pairs per thread after the planes (8-byte aligned)
-    f32x2* fold_tot = (f32x2*)(smem + ((2 * SW * SH + SH * TILE_W + 1) & ~1)) +
-                      (threadIdx.y * TILE_W + threadIdx.x);
-    const int ub = tx_ * TILE_W, vb = ty_ * TH;
+    f32x2* fold_tot = (f32x2*)(smem + ((2 * SW * SH + SH * TW + 1) & ~1)) + tid;
 
     // stage the tile + halo (Sec. 3.2, first item: the range image): warp w
     // takes halo rows w, w + NW, ..., its lanes the columns in passes of 32.
@@ -731,10 +747,10 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
 #pragma unroll
         for (int pass = 0; pass < 3; pass++) {
             const int sx = pass * 32 + lane;
-            if (pass * 32 >= SW) break;  // uniform over the warp
+            if (pass * 32 >= SWU) break;  // uniform over the warp
             const int gu = ub - halo + sx;
             float z = 0.f, c = __int_as_float(0x7f800000);
-            if (sx < SW && row_in && gu >= 0 && gu < W) {
+            if (sx < SWU && row_in && gu >= 0 && gu < W) {
                 float d;
                 if (FMT == 0) {
                     d = __ldg(depth + (size_t)gv * W + gu);
@@ -752,7 +768,7 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
                     c = 1.f;
                 }
             }
-            if (sx < SW) {
+            if (sx < SWU) {
                 tz[sy * SW + sx] = z;
                 tcv[sy * SW + sx] = c;
             }
@@ -764,23 +780,25 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         // bits col + halo - r0 ... col + halo + r0 of the row: start <= 31 + halo <= 55
         const int start = lane + halo - r0;
         const unsigned long long w = (lo >> start) | (start > 0 ? hi << (64 - start) : 0ull);
-        rcnt[sy * TILE_W + lane] = __popcll(w & seg);
+        if (lane < TW) rcnt[sy * TW + lane] = __popcll(w & seg);
     }
     __syncthreads();
 
     // the thread's pixel (tile column pxl, row pyl) and its lane in the group
     int pxl, pyl, sub = 0;
-    if constexpr (G == 1) {
+    if constexpr (G == 1 && STRIPS) {
+        pxl = tid & (TW - 1);
+        pyl = tid >> lg;
+    } else if constexpr (G == 1) {
         pxl = threadIdx.x;
         pyl = threadIdx.y;
     } else {
-        const int t = threadIdx.y * TILE_W + threadIdx.x;
-        pxl = (t / G) % TILE_W;
-        pyl = t / G / TILE_W;
-        sub = t % G;
+        pxl = (tid / G) % TILE_W;
+        pyl = tid / G / TILE_W;
+        sub = tid % G;
     }
     const int u0 = ub + pxl, v0 = vb + pyl;
-    const bool inside = u0 < W && v0 < H;
+    const bool inside = u0 < W && v0 < vend;
     // no barrier follows in this function; lane groups keep every lane for
     // their shuffles (a pixel outside the image computes on staged values and
     // stores nothing)
@@ -804,8 +822,8 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
     // ---- window count (row segments counted above)
     int cnt = 0;
     if (ok) {
-        const int* rc = rcnt + (pyl + halo) * TILE_W + pxl;
-        for (int dv = -r0; dv <= r0; dv += s) cnt += rc[dv * TILE_W];
+        const int* rc = rcnt + (pyl + halo) * TW + pxl;
+        for (int dv = -r0; dv <= r0; dv += s) cnt += rc[dv * TW];
         ok = cnt >= cfg.min_window;
     }
 
@@ -866,16 +884,26 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         const float esc2 = (sig * tz0) * (sig * tz0);
         const float wcr = (REJECT && !(esc2 <= thr)) ? 0.f : wc;
 
+        // The window's row addresses are the same in every iteration.  Made opaque
+        // here, they are computed again instead of all being kept in registers,
+        // which spilled for small windows (GB300, 640 x 480, T = 5, a frame
+        // batched: r = 2 94.3 -> 88.4 us, r = 14 2.404 -> 2.314 ms alone).
+        if (STRIPS) asm volatile("" : "+r"(SW));
+        const float *zc = tz + cidx, *cc = tcv + cidx;
         Moments2 m, comp;
         zero(m);
         zero(comp);
+        auto state_first = [&](float za, float zb, float ca, float cb, f32x2 DU, f32x2 DV) {
+            return pair_state<REJECT, true>(k, za, zb, ca, cb, DU, mul2(DV, CY0), mul2(DV, CY1), mul2(DV, CY2), thr);
+        };
+        auto state_later = [&](float za, float zb, float ca, float cb, f32x2 DU, f32x2 DV) {
+            return pair_state<REJECT, false>(k, za, zb, ca, cb, DU, mul2(DV, CY0), mul2(DV, CY1), mul2(DV, CY2), thr);
+        };
         auto first = [&](float za, float zb, float ca, float cb, f32x2 DU, f32x2 DV) {
-            visit2<REJECT, KAHAN, true>(m, comp, k, za, zb, ca, cb, DU, mul2(DV, CY0), mul2(DV, CY1),
-                                        mul2(DV, CY2), thr);
+            add_pair<KAHAN, true>(m, comp, state_first(za, zb, ca, cb, DU, DV));
         };
         auto later = [&](float za, float zb, float ca, float cb, f32x2 DU, f32x2 DV) {
-            visit2<REJECT, KAHAN, false>(m, comp, k, za, zb, ca, cb, DU, mul2(DV, CY0), mul2(DV, CY1),
-                                         mul2(DV, CY2), thr);
+            add_pair<KAHAN, false>(m, comp, state_later(za, zb, ca, cb, DU, DV));
         };
         // fold the J^T W J partials after every PC_FOLD_ROWS pairs of rows: the
         // first fold starts the totals, the centre row's partial joins at the end
@@ -963,13 +991,20 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
 // one CTA per SM instead of spilling.
 #define PC_BLOCKS_OF(PREC) (((PREC) & PREC_KAHAN) ? 1 : PC_MIN_BLOCKS)
 
-// One CTA per tile; grid row y computes tile row ty0 + y of the frame (a band
-// of tile rows when ty0 > 0 or the grid is shorter than the frame).
-template <int RW, bool REJECT, int PREC, int TH, int G, int RS>
+// One CTA per tile of the band of pixel rows row0 .. row1 - 1 of the frame.
+template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS>
 __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH * G)))
-    k_fit(FrameArgs f, FitConfig cfg, int ty0) {
+    k_fit(FrameArgs f, FitConfig cfg, int row0, int row1) {
     extern __shared__ float smem[];
-    fit_tile<RW, REJECT, PREC, TH, G, RS>(f, cfg, blockIdx.x, ty0 + blockIdx.y, smem);
+    if constexpr (STRIPS) {
+        const TilePos p = tile_pos(tiling_of(row1 - row0, f.W, TH, true), blockIdx.x, TH);
+        fit_tile<RW, REJECT, PREC, TH, G, RS, true>(f, cfg, p.ub, row0 + p.vb, p.lg, row1, smem);
+    } else {
+        // a two-dimensional grid, so that nothing but the block and thread index
+        // says where a pixel lies
+        fit_tile<RW, REJECT, PREC, TH, G, RS, false>(f, cfg, blockIdx.x * TILE_W, row0 + blockIdx.y * TH, 5, row1,
+                                                            smem);
+    }
 }
 
 // Persistent form over many frames: the CTAs take (frame, tile) items from a
@@ -993,9 +1028,9 @@ __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH
             const int mid = (lo + hi + 1) >> 1;
             if (fr[mid].tile_begin <= t) lo = mid; else hi = mid - 1;
         }
-        const int local = t - fr[lo].tile_begin, tiles_x = fr[lo].tiles_x;
-        const int ty_ = local / tiles_x;
-        fit_tile<RW, REJECT, PREC, TH, G, RS>(fr[lo].f, cfg, local - ty_ * tiles_x, ty_, smem);
+        const int H = fr[lo].f.H;
+        const TilePos p = tile_pos(tiling_of(H, fr[lo].f.W, TH, G == 1), t - fr[lo].tile_begin, TH);
+        fit_tile<RW, REJECT, PREC, TH, G, RS, G == 1>(fr[lo].f, cfg, p.ub, p.vb, p.lg, H, smem);
         __syncthreads();  // shared memory and s_tile are reused by the next tile
         if (threadIdx.x == 0 && threadIdx.y == 0) s_tile = (int)(gridDim.x + atomicAdd(next_tile, 1u));
         __syncthreads();
@@ -1008,7 +1043,7 @@ __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH
 template <int PREC, int TH, int G>
 size_t variant_smem_bytes(const FitConfig& cfg) {
     constexpr bool FOLD = G == 1 && (PREC & PREC_KAHAN) == 0;
-    return fit_smem_bytes(cfg, TH, FOLD ? TILE_W * TH : 0);
+    return fit_smem_bytes(cfg, TH, G == 1, FOLD ? TILE_W * TH : 0);
 }
 
 // Kernels whose dynamic shared memory exceeds the default 48 KB opt in on the
@@ -1023,17 +1058,27 @@ cudaError_t allow_smem(K kernel, size_t smem) {
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>
 cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t stream, int ty0, int ty1) {
     const dim3 block(TILE_W, TH * G);
-    const dim3 grid((f.W + TILE_W - 1) / TILE_W, ty1 - ty0);
+    const int row0 = ty0 * TH, row1 = ty1 * TH < f.H ? ty1 * TH : f.H;
+    const Tiling tl = tiling_of(row1 - row0, f.W, TH, G == 1);
+    const dim3 strips(tl.full + tl.n16 + tl.n8), columns(tl.cols, (row1 - row0 + TH - 1) / TH);
     const size_t smem = variant_smem_bytes<PREC, TH, G>(cfg);
-    cudaError_t e;
-    if (cfg.reject) {
-        if ((e = allow_smem(k_fit<RW, true, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
-        k_fit<RW, true, PREC, TH, G, RS><<<grid, block, smem, stream>>>(f, cfg, ty0);
-    } else {
-        if ((e = allow_smem(k_fit<RW, false, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
-        k_fit<RW, false, PREC, TH, G, RS><<<grid, block, smem, stream>>>(f, cfg, ty0);
+    auto launch = [&](auto* kernel, dim3 grid) {
+        const cudaError_t e = allow_smem(kernel, smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, block, smem, stream>>>(f, cfg, row0, row1);
+        return cudaGetLastError();
+    };
+    // Plain FP32 windows of 5 to 7 samples' radius without strips keep the form
+    // that knows the tile's shape when compiled, whose loop needs no more
+    // registers than it has (GB300, 640 x 480 frames alone: r = 6 3.577 against
+    // 3.640 ms for eight, the 37 x 37 patch 3.622 against 3.690, r = 7 4.621
+    // against 4.638); elsewhere the form with strips is as fast or faster.
+    if constexpr (PREC == 0 && G == 1 && RW / RS >= 5 && RW / RS <= 7) {
+        if (!cfg.reject && tl.n16 + tl.n8 == 0) return launch(k_fit<RW, false, PREC, TH, G, RS, false>, columns);
     }
-    return cudaGetLastError();
+    const dim3 grid = G == 1 ? strips : columns;
+    return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, G == 1>, grid)
+                      : launch(k_fit<RW, false, PREC, TH, G, RS, G == 1>, grid);
 }
 
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>

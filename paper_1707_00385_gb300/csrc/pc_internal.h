@@ -3,6 +3,12 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#ifdef __CUDACC__
+#define PC_HD __host__ __device__
+#else
+#define PC_HD
+#endif
+
 namespace pcurv {
 
 // Pinhole intrinsics (pixels) and their reciprocals.
@@ -59,17 +65,74 @@ inline int halo_of(const FitConfig& c) { return c.r > c.rn ? c.r : c.rn; }
 // shared memory, as one pair of floats per thread (fit_tile, fold_rows).
 constexpr int FOLD_SUMS = 20;
 
-// Z and c planes of the tile + halo, per-row valid counts and, for
-// fold_threads > 0, the folded totals of that many threads (8-byte aligned).
-inline size_t fit_smem_bytes(const FitConfig& c, int th, int fold_threads = 0) {
-    const int h = halo_of(c);
-    const size_t planes = (size_t)(TILE_W + 2 * h) * (th + 2 * h) * 2 * sizeof(float) +
-                          (size_t)(th + 2 * h) * TILE_W * sizeof(int);
-    return (planes + 7) / 8 * 8 + (size_t)fold_threads * FOLD_SUMS * 8;
+// Tiles of a band of `rows` pixel rows of a frame W pixels wide, for CTAs of
+// 32 x th threads.  Lane groups (strips = false) cover the width with 32-pixel
+// columns.  One thread per pixel: the columns that fill 32 pixels, then the
+// rest of the width, in a last column or, where that takes fewer tiles, in
+// strips 16 and 8 pixels wide whose tiles are 2 and 4 times as tall, so that a
+// ragged width leaves the threads of at most 7 pixel columns idle instead of
+// 31.  The kernels' time goes with the warps that run, whether or not their
+// threads have a pixel.  GB300, with the rule that chooses the tile height:
+// one 323 x 241 frame (r = 5, T = 5) 127.0 -> 110.8 us, one 682 x 579 frame
+// (r = 2, rejection) 246 -> 166 us, 27 frames of 122 x 64, 792 x 709 and
+// 64 x 52 in one batch (r = 9) 18.84 -> 18.63 ms; widths that are a multiple of
+// 32 have no strips.  Queue order: columns (row by row of tiles), 16-wide
+// strip, 8-wide strip.
+struct Tiling {
+    int cols;          // 32-pixel columns
+    int full, n16, n8; // tiles in the columns and in the two strips
+};
+struct TilePos {
+    int ub, vb;        // first pixel (vb from the band's first row)
+    int lg;            // log2 of the width: 5, 4 or 3; the height is (32 th) >> lg
+};
+PC_HD inline Tiling tiling_of(int rows, int W, int th, bool strips) {
+    Tiling t;
+    const int rem = W % TILE_W, rows_t = (rows + th - 1) / th;
+    t.cols = W / TILE_W;
+    t.n16 = rem > 8 ? (rows + 2 * th - 1) / (2 * th) : 0;
+    t.n8 = (rem > 0 && rem <= 8) || rem > 16 ? (rows + 4 * th - 1) / (4 * th) : 0;
+    if (rem > 0 && (!strips || rem > 24 || t.n16 + t.n8 >= rows_t)) {
+        t.cols++;
+        t.n16 = t.n8 = 0;
+    }
+    t.full = t.cols * rows_t;
+    return t;
+}
+PC_HD inline TilePos tile_pos(const Tiling& t, int i, int th) {
+    if (i < t.full) {
+        const int row = i / t.cols;
+        return TilePos{(i - row * t.cols) * TILE_W, row * th, 5};
+    }
+    i -= t.full;
+    if (i < t.n16) return TilePos{t.cols * TILE_W, i * 2 * th, 4};
+    return TilePos{t.cols * TILE_W + (t.n16 > 0 ? 16 : 0), (i - t.n16) * 4 * th, 3};
+}
+inline long long tiles_of(int rows, int W, int variant) {
+    const Tiling t = tiling_of(rows, W, tile_h_of(variant), lanes_of(variant) == 1);
+    return (long long)t.full + t.n16 + t.n8;
 }
 
-inline long long tiles_of(int H, int W, int th) {
-    return (long long)((W + TILE_W - 1) / TILE_W) * ((H + th - 1) / th);
+// Row pitch of the staged planes of a tile tw pixels wide.  A warp of a strip
+// tile spans 2 rows of 16 or 4 rows of 8 pixels: the pitch is padded so that
+// those rows fall into different shared-memory banks.
+PC_HD inline int tile_pitch(int tw, int halo) {
+    const int sw = tw + 2 * halo;
+    return tw == 16 ? sw + (48 - sw % 32) % 32 : tw == 8 ? sw + (24 - sw % 16) % 16 : sw;
+}
+
+// Z and c planes of the tile + halo, per-row valid counts (the largest of the
+// tile shapes the variant uses) and, for fold_threads > 0, the folded totals
+// of that many threads (8-byte aligned).
+inline size_t fit_smem_bytes(const FitConfig& c, int th, bool strips, int fold_threads = 0) {
+    const int h = halo_of(c);
+    size_t planes = 0;
+    for (int tw = TILE_W; tw >= (strips ? 8 : TILE_W); tw /= 2) {
+        const int rows = TILE_W * th / tw + 2 * h;
+        const size_t b = (size_t)tile_pitch(tw, h) * rows * 2 * sizeof(float) + (size_t)rows * tw * sizeof(int);
+        planes = b > planes ? b : planes;
+    }
+    return (planes + 7) / 8 * 8 + (size_t)fold_threads * FOLD_SUMS * 8;
 }
 
 // One frame: caller-owned device buffers, size and intrinsics.
@@ -89,8 +152,8 @@ struct FrameArgs {
 // A frame of a batch and its place in the flattened tile queue.
 struct BatchFrame {
     FrameArgs f;
-    int tiles_x;     // tiles per row of this frame
     int tile_begin;  // first queue index of this frame
+    int pad;
 };
 
 // Device-resident batch table: header followed by nframes descriptors.

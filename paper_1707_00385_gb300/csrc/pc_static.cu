@@ -106,7 +106,6 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
     // bits as the 32 x 4 tiles its heuristic may pick instead)
     int v = pcurv::ctx_forced_variant(ctx);
     if (v < 0 || !ops->batch[v]) v = 0;
-    const int th = pcurv::tile_h_of(v);
     long long total = 0;
     int live = 0;
     for (int i = 0; i < n; i++) {
@@ -114,7 +113,7 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
         if (f.H < 0 || f.W < 0 || f.H > PC_MAX_DIM || f.W > PC_MAX_DIM) return PC_ERR_INVALID_ARG;
         if (f.H == 0 || f.W == 0) continue;
         if (!ok_intrinsics(f) || !ok_buffers(f)) return PC_ERR_INVALID_ARG;
-        total += pcurv::tiles_of(f.H, f.W, th);
+        total += pcurv::tiles_of(f.H, f.W, v);
         live++;
     }
     if (live == 0) return PC_OK;
@@ -147,9 +146,8 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
         d.f = pcurv::FrameArgs{f.depth, f.H, f.W,
                                pcurv::Camera{f.fx, f.fy, f.cx, f.cy, 1.f / f.fx, 1.f / f.fy},
                                f.k1, f.k2, f.normal, nullptr, nullptr};
-        d.tiles_x = (f.W + pcurv::TILE_W - 1) / pcurv::TILE_W;
         d.tile_begin = begin;
-        begin += d.tiles_x * ((f.H + th - 1) / th);
+        begin += (int)pcurv::tiles_of(f.H, f.W, v);
     }
     t->nframes = live;
     t->total_tiles = begin;

@@ -72,6 +72,19 @@
 #ifndef PC_FOLD_ROWS
 #define PC_FOLD_ROWS 3
 #endif
+// Window radius (in samples) from which the unrolled kernels form each pair's
+// state one pair ahead (for_each_pair_ahead), in the batch and the per-frame
+// form.  Measured on both sides of the lines (GB300, 640 x 480, T = 5, time
+// without over time with it): batch r = 3 .. 6 0.997 to 1.005, r = 7 1.018,
+// r = 8 .. 12 1.015 to 1.020; alone r = 5 1.000, r = 7 0.983, r = 8 1.009,
+// r = 9 1.011, r = 11 1.031, r = 12 1.025.  32 frames of 640 x 480, r = 7, in
+// one launch: 18.62 -> 18.29 ms.
+#ifndef PC_AHEAD_BATCH
+#define PC_AHEAD_BATCH 7
+#endif
+#ifndef PC_AHEAD_FRAME
+#define PC_AHEAD_FRAME 8
+#endif
 #define PC_STR(x) #x
 #define PC_UNROLL(n) _Pragma(PC_STR(unroll n))
 
@@ -531,6 +544,47 @@ __device__ __forceinline__ void for_each_pair(const float* zc, const float* cc, 
     for_each_pair<RW, RS>(zc, cc, SW, r, s, f, [](int) {});
 }
 
+// for_each_pair with the state of the next pair formed before the sums of the
+// present one, so that the loads, the reciprocal and the chain of dependent
+// operations behind a weight have the 26 sums of another pair to hide in.
+// state(za, zb, ca, cb, DU, DV) forms a pair's state, sums(state) adds it.  A
+// row's last pair is added before the next row's first one is formed.  The
+// same operations in the same order on every sum: the same bits.
+template <int RW, int RS = 1, typename S, typename F, typename E>
+__device__ __forceinline__ void for_each_pair_ahead(const float* zc, const float* cc, int SW, S&& state, F&& sums,
+                                                    E&& row_end) {
+    constexpr int R0 = (RW / RS) * RS;
+    const f32x2 STEP = pack((float)RS, -(float)RS);
+    int row = 0;
+    for (int dv = -R0; dv < 0; dv += RS, row++) {
+        const float *za = zc + dv * SW, *zb = zc - dv * SW;
+        const float *ca = cc + dv * SW, *cb = cc - dv * SW;
+        const f32x2 DV = pack((float)dv, -(float)dv);
+        f32x2 DU = pack(-(float)R0, (float)R0);
+        auto p = state(za[-R0], zb[R0], ca[-R0], cb[R0], DU, DV);
+#pragma unroll
+        for (int du = -R0 + RS; du <= R0; du += RS) {
+            DU = add2(DU, STEP);
+            const auto next = state(za[du], zb[-du], ca[du], cb[-du], DU, DV);
+            sums(p);
+            p = next;
+        }
+        sums(p);
+        row_end(row);
+    }
+    const f32x2 DV0 = 0ull;
+    f32x2 DU = pack(-(float)R0, (float)R0);
+    auto p = state(zc[-R0], zc[R0], cc[-R0], cc[R0], DU, DV0);
+#pragma unroll
+    for (int du = -R0 + RS; du < 0; du += RS) {
+        DU = add2(DU, STEP);
+        const auto next = state(zc[du], zc[-du], cc[du], cc[-du], DU, DV0);
+        sums(p);
+        p = next;
+    }
+    sums(p);
+}
+
 // The share of one lane of a group of G lanes that computes one pixel
 // together: the window splits into row units, units 0 .. r0/s - 1 being the
 // rows dv = -r0 + k s (each point paired with its reflection (-du, -dv)) and
@@ -695,7 +749,8 @@ __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_r
 // (reduce_lanes) before each solve, which every lane of the group repeats;
 // only the order of the moment sums differs from G = 1.
 // STRIPS: the tile may be a strip (Tiling), else 32 x TH.
-template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS>
+// BATCH: the caller is the persistent kernel.
+template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS, bool BATCH>
 __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cfg, int ub, int vb, int lg, int vend,
                                          float* smem) {
     constexpr bool KAHAN = (PREC & PREC_KAHAN) != 0;
@@ -703,6 +758,8 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
     constexpr int NW = TH * G;  // warps of the CTA
     // fold the J^T W J sums row by row (one thread per pixel, plain sums)
     constexpr bool FOLD = G == 1 && !KAHAN;
+    // form each pair's state one pair ahead
+    constexpr bool AHEAD = FOLD && RW / RS >= (BATCH ? PC_AHEAD_BATCH : PC_AHEAD_FRAME);
     static_assert(G == 1 || G == 2 || G == 4 || G == 8, "lanes per pixel");
     static_assert(G == 1 || (!KAHAN && FMT == 0), "lane groups run the plain FP32 form");
     static_assert(G == 1 || RW == 0 || RS == 1, "lane groups with a compile-time window are dense");
@@ -926,7 +983,11 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         if (it == 0) {
             // A = B = C = 0 here: the cheaper first-iteration form
             if constexpr (G == 1) {
-                for_each_pair<RW, RS>(zc, cc, SW, r, s, first, fold_first);
+                if constexpr (AHEAD)
+                    for_each_pair_ahead<RW, RS>(
+                        zc, cc, SW, state_first, [&](const PairState& p) { add_pair<false, true>(m, comp, p); }, fold_first);
+                else
+                    for_each_pair<RW, RS>(zc, cc, SW, r, s, first, fold_first);
                 if (folded) fold_finish<true>(m, fold_tot, NT);
             } else {
                 for_each_pair_lanes<RW, G>(zc, cc, SW, r, s, sub, first);
@@ -934,7 +995,11 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
             first_iteration_sums(m, comp);
         } else {
             if constexpr (G == 1) {
-                for_each_pair<RW, RS>(zc, cc, SW, r, s, later, fold_later);
+                if constexpr (AHEAD)
+                    for_each_pair_ahead<RW, RS>(
+                        zc, cc, SW, state_later, [&](const PairState& p) { add_pair<false, false>(m, comp, p); }, fold_later);
+                else
+                    for_each_pair<RW, RS>(zc, cc, SW, r, s, later, fold_later);
                 if (folded) fold_finish<false>(m, fold_tot, NT);
             } else {
                 for_each_pair_lanes<RW, G>(zc, cc, SW, r, s, sub, later);
@@ -998,11 +1063,11 @@ __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH
     extern __shared__ float smem[];
     if constexpr (STRIPS) {
         const TilePos p = tile_pos(tiling_of(row1 - row0, f.W, TH, true), blockIdx.x, TH);
-        fit_tile<RW, REJECT, PREC, TH, G, RS, true>(f, cfg, p.ub, row0 + p.vb, p.lg, row1, smem);
+        fit_tile<RW, REJECT, PREC, TH, G, RS, true, false>(f, cfg, p.ub, row0 + p.vb, p.lg, row1, smem);
     } else {
         // a two-dimensional grid, so that nothing but the block and thread index
         // says where a pixel lies
-        fit_tile<RW, REJECT, PREC, TH, G, RS, false>(f, cfg, blockIdx.x * TILE_W, row0 + blockIdx.y * TH, 5, row1,
+        fit_tile<RW, REJECT, PREC, TH, G, RS, false, false>(f, cfg, blockIdx.x * TILE_W, row0 + blockIdx.y * TH, 5, row1,
                                                             smem);
     }
 }
@@ -1030,7 +1095,7 @@ __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH
         }
         const int H = fr[lo].f.H;
         const TilePos p = tile_pos(tiling_of(H, fr[lo].f.W, TH, G == 1), t - fr[lo].tile_begin, TH);
-        fit_tile<RW, REJECT, PREC, TH, G, RS, G == 1>(fr[lo].f, cfg, p.ub, p.vb, p.lg, H, smem);
+        fit_tile<RW, REJECT, PREC, TH, G, RS, G == 1, true>(fr[lo].f, cfg, p.ub, p.vb, p.lg, H, smem);
         __syncthreads();  // shared memory and s_tile are reused by the next tile
         if (threadIdx.x == 0 && threadIdx.y == 0) s_tile = (int)(gridDim.x + atomicAdd(next_tile, 1u));
         __syncthreads();

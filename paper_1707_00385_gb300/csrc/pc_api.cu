@@ -233,8 +233,13 @@ struct OpsTable {
 
 }  // namespace
 
+// Kernels of compensated sums.
+static const KernelOps* kahan_ops(const FitConfig& cfg, int format) {
+    return cfg.r / cfg.stride >= COMP_MIN_RADIUS ? ops_compensated(format) : ops_precision(1, format);
+}
+
 const KernelOps* select_ops(const FitConfig& cfg) {
-    if (cfg.kahan) return ops_precision(1, 0);
+    if (cfg.kahan) return kahan_ops(cfg, 0);
     static const OpsTable table;  // built once (thread-safe initialisation)
     const bool dense = cfg.stride == 1 && cfg.r >= 1 && cfg.r <= 12;
     if (cfg.r == SPARSE_RADIUS && cfg.stride == SPARSE_STRIDE) return &table.ops[13];
@@ -246,7 +251,7 @@ const KernelOps* select_packed_ops(const FitConfig& cfg, int format) {
         const KernelOps* k = format == 1 ? ops_packed_f16(cfg.r) : format == 2 ? ops_packed_bf16(cfg.r) : nullptr;
         if (k) return k;
     }
-    return ops_precision(cfg.kahan, format);
+    return cfg.kahan ? kahan_ops(cfg, format) : ops_precision(0, format);
 }
 
 const FitConfig& ctx_config(const pc_ctx* ctx) { return ctx->cfg; }

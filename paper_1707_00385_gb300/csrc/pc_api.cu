@@ -7,6 +7,7 @@
 #include <cstring>
 #include <new>
 
+#include <cuda.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/pcurv.h"
@@ -127,6 +128,51 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// The device pointers of one call.  A pointer inside an allocation that holds
+// another pointer of the call needs no query of its own: a batch of frames cut
+// from a few allocations asks the driver a few times instead of four times a
+// frame.  An allocation counts when its last byte is a device pointer too.
+// Nothing is kept from one call for the next.
+class DevicePtrs {
+  public:
+    bool operator()(const void* p) {
+        const uintptr_t a = (uintptr_t)p;
+        for (int i = 0; i < used_; i++)
+            if (a >= lo_[i] && a < hi_[i]) return true;
+        if (!is_device_ptr(p)) return false;
+        CUdeviceptr base = 0;
+        size_t size = 0;
+        const AddressRange range = address_range();
+        if (range && range(&base, &size, (CUdeviceptr)a) == CUDA_SUCCESS && size > 0 && a >= base && a - base < size &&
+            is_device_ptr((const void*)(base + size - 1))) {
+            const int i = used_ < MAX ? used_++ : next_++ % MAX;
+            lo_[i] = base;
+            hi_[i] = base + size;
+        }
+        return true;
+    }
+
+  private:
+    typedef CUresult(CUDAAPI* AddressRange)(CUdeviceptr*, size_t*, CUdeviceptr);
+    // cuMemGetAddressRange, looked up through the runtime (nullptr: every pointer is queried)
+    static AddressRange address_range() {
+        static const AddressRange f = [] {
+            void* fn = nullptr;
+            cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+            if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) !=
+                cudaSuccess) {
+                cudaGetLastError();
+                return (AddressRange) nullptr;
+            }
+            return found == cudaDriverEntryPointSuccess ? (AddressRange)fn : (AddressRange) nullptr;
+        }();
+        return f;
+    }
+    static constexpr int MAX = 8;
+    uintptr_t lo_[MAX], hi_[MAX];
+    int used_ = 0, next_ = 0;
+};
+
 pc_status check_params(const pc_params& p) {
     if (!(finite_f(p.k) && p.k > 0.f)) return PC_ERR_INVALID_ARG;
     if (p.reject != 0 && p.reject != 1) return PC_ERR_INVALID_ARG;
@@ -157,13 +203,16 @@ bool valid_intrinsics(float fx, float fy, float cx, float cy) {
 }
 
 // Device buffers of one frame: present, aligned, on the device.
-pc_status check_buffers(const float* depth, const float* k1, const float* k2, const float* normal) {
+template <typename Check>
+pc_status check_buffers(const float* depth, const float* k1, const float* k2, const float* normal, Check& on_device) {
     if (!depth || !k1 || !k2) return PC_ERR_INVALID_ARG;
     if (!aligned4(depth) || !aligned4(k1) || !aligned4(k2) || !aligned4(normal)) return PC_ERR_INVALID_ARG;
-    if (!is_device_ptr(depth) || !is_device_ptr(k1) || !is_device_ptr(k2) ||
-        (normal && !is_device_ptr(normal)))
+    if (!on_device(depth) || !on_device(k1) || !on_device(k2) || (normal && !on_device(normal)))
         return PC_ERR_INVALID_ARG;
     return PC_OK;
+}
+pc_status check_buffers(const float* depth, const float* k1, const float* k2, const float* normal) {
+    return check_buffers(depth, k1, k2, normal, is_device_ptr);
 }
 
 void release_batch(BatchScratch& b) {
@@ -767,13 +816,14 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
     long long queue = 0;              // 32 x 8 tiles without strips: bounds both of the totals' halves
     long long total = 0, total4 = 0;  // tiles of 256 and of 128 threads
     int live = 0;
+    DevicePtrs on_device;
     for (int i = 0; i < n; i++) {
         const pc_frame& fr = frames[i];
         pc_status st = check_image(fr.H, fr.W);
         if (st != PC_OK) return st;
         if (fr.H == 0 || fr.W == 0) continue;
         if (!valid_intrinsics(fr.fx, fr.fy, fr.cx, fr.cy)) return PC_ERR_INVALID_ARG;
-        if ((st = check_buffers(fr.depth, fr.k1, fr.k2, fr.normal)) != PC_OK) return st;
+        if ((st = check_buffers(fr.depth, fr.k1, fr.k2, fr.normal, on_device)) != PC_OK) return st;
         queue += (long long)((fr.W + 31) / 32) * ((fr.H + 7) / 8);
         total += pcurv::tiles_of(fr.H, fr.W, 0);
         total4 += pcurv::tiles_of(fr.H, fr.W, 1);
@@ -838,12 +888,12 @@ pc_status pc_compute_batch(pc_ctx* ctx, const pc_frame* frames, int n, void* str
 }
 
 // Device buffers of one packed frame: present, aligned, on the device.
-static pc_status check_packed_frame(const pc_packed_frame& f) {
-    if (!f.packed || !f.tile_base || !aligned2(f.packed) || !aligned4(f.tile_base) || !is_device_ptr(f.packed) ||
-        !is_device_ptr(f.tile_base))
+static pc_status check_packed_frame(const pc_packed_frame& f, DevicePtrs& on_device) {
+    if (!f.packed || !f.tile_base || !aligned2(f.packed) || !aligned4(f.tile_base) || !on_device(f.packed) ||
+        !on_device(f.tile_base))
         return PC_ERR_INVALID_ARG;
-    if (!f.k1 || !f.k2 || !aligned4(f.k1) || !aligned4(f.k2) || !aligned4(f.normal) || !is_device_ptr(f.k1) ||
-        !is_device_ptr(f.k2) || (f.normal && !is_device_ptr(f.normal)))
+    if (!f.k1 || !f.k2 || !aligned4(f.k1) || !aligned4(f.k2) || !aligned4(f.normal) || !on_device(f.k1) ||
+        !on_device(f.k2) || (f.normal && !on_device(f.normal)))
         return PC_ERR_INVALID_ARG;
     return PC_OK;
 }
@@ -855,13 +905,14 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
         return PC_ERR_INVALID_ARG;
     long long total = 0;  // 32 x 8 tiles
     int live = 0;
+    DevicePtrs on_device;
     for (int i = 0; i < n; i++) {
         const pc_packed_frame& fr = frames[i];
         pc_status st = check_image(fr.H, fr.W);
         if (st != PC_OK) return st;
         if (fr.H == 0 || fr.W == 0) continue;
         if (!valid_intrinsics(fr.fx, fr.fy, fr.cx, fr.cy)) return PC_ERR_INVALID_ARG;
-        if ((st = check_packed_frame(fr)) != PC_OK) return st;
+        if ((st = check_packed_frame(fr, on_device)) != PC_OK) return st;
         total += (long long)((fr.W + 31) / 32) * ((fr.H + 7) / 8);
         live++;
     }

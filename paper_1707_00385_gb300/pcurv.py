@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "lib", "libpcurv.so")
@@ -57,6 +58,10 @@ class pc_packed_frame(ctypes.Structure):
         ("fx", ctypes.c_float), ("fy", ctypes.c_float), ("cx", ctypes.c_float), ("cy", ctypes.c_float),
         ("k1", ctypes.c_void_p), ("k2", ctypes.c_void_p), ("normal", ctypes.c_void_p),
     ]
+
+
+_FRAME = struct.Struct("=QiiffffQQQ")          # pc_frame
+_PACKED_FRAME = struct.Struct("=QQiiffffQQQ")  # pc_packed_frame
 
 
 class PcError(RuntimeError):
@@ -242,10 +247,52 @@ def pc_fp32_peak_kernel(blocks, iters, packed, sink, sink_len, stream):
 # ---- torch convenience wrapper ----------------------------------------------
 
 def _stream_handle(stream):
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return stream.cuda_stream
+    # torch.cuda.current_stream() without building its Stream object
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _frame_array(frames):
+    """A ctypes array of pc_frame for (depth, intrinsics, k1, k2, normal) tuples.
+
+    The descriptors are written with one struct call each (256 frames on the
+    GB300's host: 0.13 ms, against 0.33 ms through ctypes constructors), which
+    a value out of a C type's range refuses; ctypes then converts it, and the
+    library judges it."""
+    buf = bytearray(_FRAME.size * len(frames))
+    try:
+        for i, (d, (fx, fy, cx, cy), a, b, n) in enumerate(frames):
+            H, W = d.shape
+            _FRAME.pack_into(buf, i * _FRAME.size, d.data_ptr(), H, W, fx, fy, cx, cy, a.data_ptr(), b.data_ptr(),
+                             0 if n is None else n.data_ptr())
+    except (OverflowError, struct.error):
+        arr = (pc_frame * len(frames))()
+        for i, (d, intr, a, b, n) in enumerate(frames):
+            H, W = d.shape
+            arr[i] = pc_frame(d.data_ptr(), H, W, *map(float, intr), a.data_ptr(), b.data_ptr(),
+                              n.data_ptr() if n is not None else None)
+        return arr
+    return (pc_frame * len(frames)).from_buffer(buf)
+
+
+def _packed_frame_array(frames):
+    """The same of pc_packed_frame for (packed, tile_base, intrinsics, k1, k2, normal) tuples."""
+    buf = bytearray(_PACKED_FRAME.size * len(frames))
+    try:
+        for i, (q, base, (fx, fy, cx, cy), a, b, n) in enumerate(frames):
+            H, W = q.shape
+            _PACKED_FRAME.pack_into(buf, i * _PACKED_FRAME.size, q.data_ptr(), base.data_ptr(), H, W, fx, fy, cx, cy,
+                                    a.data_ptr(), b.data_ptr(), 0 if n is None else n.data_ptr())
+    except (OverflowError, struct.error):
+        arr = (pc_packed_frame * len(frames))()
+        for i, (q, base, intr, a, b, n) in enumerate(frames):
+            H, W = q.shape
+            arr[i] = pc_packed_frame(q.data_ptr(), base.data_ptr(), H, W, *map(float, intr), a.data_ptr(),
+                                     b.data_ptr(), n.data_ptr() if n is not None else None)
+        return arr
+    return (pc_packed_frame * len(frames)).from_buffer(buf)
 
 
 class Curvature:
@@ -287,17 +334,17 @@ class Curvature:
             raise ValueError("depth must be a 2-D float32 CUDA tensor")
         depth = depth.contiguous()
         H, W = depth.shape
-        if k1 is None:
-            k1 = torch.empty((H, W), dtype=torch.float32, device=depth.device)
-        if k2 is None:
-            k2 = torch.empty((H, W), dtype=torch.float32, device=depth.device)
-        if want_normal and normal is None:
-            normal = torch.empty((H, W, 3), dtype=torch.float32, device=depth.device)
-        for t in (k1, k2) + ((normal,) if normal is not None else ()):
-            if not t.is_contiguous() or t.dtype != torch.float32:
+        for t in (k1, k2, normal):
+            if t is not None and (not t.is_contiguous() or t.dtype != torch.float32):
                 raise ValueError("outputs must be contiguous float32")
-        st = pc_compute(self.ctx, depth.data_ptr(), H, W, _stream_handle(stream), k1.data_ptr(),
-                        k2.data_ptr(), normal.data_ptr() if normal is not None else None)
+        if k1 is None:
+            k1 = depth.new_empty((H, W))
+        if k2 is None:
+            k2 = depth.new_empty((H, W))
+        if want_normal and normal is None:
+            normal = depth.new_empty((H, W, 3))
+        st = load().pc_compute(self.ctx, depth.data_ptr(), H, W, _stream_handle(stream), k1.data_ptr(),
+                               k2.data_ptr(), normal.data_ptr() if normal is not None else None)
         if st != PC_OK:
             raise PcError(st, "pc_compute", pc_last_error(self.ctx))
         return k1, k2, normal
@@ -356,12 +403,7 @@ class Curvature:
     def batch(self, frames, stream=None):
         """pc_compute_batch over a list of (depth, (fx, fy, cx, cy), k1, k2, normal)
         tuples of CUDA tensors (normal may be None); enqueues one persistent launch."""
-        arr = (pc_frame * max(len(frames), 1))()
-        for i, (d, intr, a, b, n) in enumerate(frames):
-            H, W = d.shape
-            arr[i] = pc_frame(d.data_ptr(), H, W, *map(float, intr), a.data_ptr(), b.data_ptr(),
-                              n.data_ptr() if n is not None else None)
-        st = pc_compute_batch(self.ctx, arr if frames else None, len(frames), _stream_handle(stream))
+        st = pc_compute_batch(self.ctx, _frame_array(frames) if frames else None, len(frames), _stream_handle(stream))
         if st != PC_OK:
             raise PcError(st, "pc_compute_batch", pc_last_error(self.ctx))
 
@@ -394,12 +436,8 @@ class Curvature:
         """pc_compute_packed_batch over a list of (packed, tile_base, (fx, fy, cx, cy),
         k1, k2, normal) tuples of CUDA tensors (the storage of pack(), all in
         format fmt; normal may be None); enqueues one persistent launch."""
-        arr = (pc_packed_frame * max(len(frames), 1))()
-        for i, (q, base, intr, a, b, n) in enumerate(frames):
-            H, W = q.shape
-            arr[i] = pc_packed_frame(q.data_ptr(), base.data_ptr(), H, W, *map(float, intr), a.data_ptr(),
-                                     b.data_ptr(), n.data_ptr() if n is not None else None)
-        st = pc_compute_packed_batch(self.ctx, arr if frames else None, len(frames), fmt, _stream_handle(stream))
+        st = pc_compute_packed_batch(self.ctx, _packed_frame_array(frames) if frames else None, len(frames), fmt,
+                                     _stream_handle(stream))
         if st != PC_OK:
             raise PcError(st, "pc_compute_packed_batch", pc_last_error(self.ctx))
 
@@ -407,12 +445,8 @@ class Curvature:
         """pc_compute_host_batch over a list of (depth, (fx, fy, cx, cy), k1, k2,
         normal) tuples of CPU float32 tensors (pinned for the copies to overlap;
         normal may be None).  Synchronise the stream before reading the outputs."""
-        arr = (pc_frame * max(len(frames), 1))()
-        for i, (d, intr, a, b, n) in enumerate(frames):
-            H, W = d.shape
-            arr[i] = pc_frame(d.data_ptr(), H, W, *map(float, intr), a.data_ptr(), b.data_ptr(),
-                              n.data_ptr() if n is not None else None)
-        st = pc_compute_host_batch(self.ctx, arr if frames else None, len(frames), _stream_handle(stream))
+        st = pc_compute_host_batch(self.ctx, _frame_array(frames) if frames else None, len(frames),
+                                   _stream_handle(stream))
         if st != PC_OK:
             raise PcError(st, "pc_compute_host_batch", pc_last_error(self.ctx))
 

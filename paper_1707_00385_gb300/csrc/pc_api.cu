@@ -322,6 +322,7 @@ cudaError_t sm_count(pc_ctx* ctx, int* sms) {
         if ((e = cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
             return e;
         ctx->sms_device = dev;
+        ctx->cfg.sms = ctx->sms;
         for (int& n : ctx->resident) n = 0;
     }
     *sms = ctx->sms;
@@ -371,15 +372,17 @@ int heuristic_variant(const pcurv::FitConfig& c, long long tiles8, long long til
 // Tile variant for one H x W image: forced, tuned, or the heuristic (one lane
 // per pixel); always one that ops has.
 cudaError_t variant_for(pc_ctx* ctx, const pcurv::KernelOps* ops, int H, int W, int* v) {
+    int sms = 0;
+    const cudaError_t e = sm_count(ctx, &sms);  // the launch, too, goes by it (FitConfig::sms)
     int choice = forced_variant(ctx);
     if (choice < 0) {
         for (const Plan& pl : ctx->plans)
             if (pl.stamp && pl.H == H && pl.W == W && plan_allows(ctx, pl.variant)) choice = pl.variant;
     }
-    if (choice < 0) {
-        int sms = 0;
-        const cudaError_t e = sm_count(ctx, &sms);
-        if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+        if (choice < 0) return e;
+        cudaGetLastError();  // not needed after all: the choice is made
+    } else if (choice < 0) {
         choice = heuristic_variant(ctx->cfg, pcurv::tiles_of(H, W, 0), pcurv::tiles_of(H, W, 1), sms);
     }
     *v = ops->fit[choice] ? choice : 0;
@@ -451,7 +454,7 @@ pc_status pc_create(float fx, float fy, float cx, float cy, int window_radius, i
     c->cam = pcurv::Camera{fx, fy, cx, cy, 1.f / fx, 1.f / fy};
     c->cfg = pcurv::FitConfig{window_radius, p.normal_radius, iterations, p.stride, 1.f / p.k,
                               p.reject, p.reject_ratio, p.det_tol, p.pivot_tol, p.min_window,
-                              p.kahan, p.fp64_solve_cond > 0.f ? 1.f / p.fp64_solve_cond : 0.f};
+                              p.kahan, p.fp64_solve_cond > 0.f ? 1.f / p.fp64_solve_cond : 0.f, 0};
     *out = c;
     return PC_OK;
 }
@@ -486,7 +489,9 @@ pc_status pc_autotune(pc_ctx* ctx, const float* depth, int H, int W, void* strea
     const pcurv::KernelOps* ops = pcurv::select_ops(ctx->cfg);
     cudaStream_t s = (cudaStream_t)stream;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    cudaError_t e;
+    int sms = 0;
+    cudaError_t e = sm_count(ctx, &sms);  // the launches go by it (FitConfig::sms)
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "pc_autotune");
     if ((e = cudaEventCreate(&e0)) != cudaSuccess || (e = cudaEventCreate(&e1)) != cudaSuccess) {
         if (e0) cudaEventDestroy(e0);
         return cuda_fail(ctx, e, "pc_autotune events");

@@ -830,8 +830,8 @@ __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_r
 // (reduce_lanes) before each solve, which every lane of the group repeats;
 // only the order of the moment sums differs from G = 1.
 // STRIPS: the tile may be a strip (Tiling), else 32 x TH.
-// BATCH: the caller is the persistent kernel.
-template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS, bool BATCH>
+// AHEAD_FROM: radius in samples from which pairs' states are formed one ahead.
+template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS, int AHEAD_FROM>
 __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cfg, int ub, int vb, int lg, int vend,
                                          float* smem) {
     constexpr bool BLOCKS = prec_blocks(PREC);                   // J^T W J compensated block by block
@@ -842,7 +842,7 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
     // fold the J^T W J sums row by row (one thread per pixel, plain sums)
     constexpr bool FOLD = G == 1 && !KAHAN && !BLOCKS;
     // form each pair's state one pair ahead
-    constexpr bool AHEAD = FOLD && RW / RS >= (BATCH ? PC_AHEAD_BATCH : PC_AHEAD_FRAME);
+    constexpr bool AHEAD = FOLD && RW / RS >= AHEAD_FROM;
     static_assert(G == 1 || G == 2 || G == 4 || G == 8, "lanes per pixel");
     static_assert(!BLOCKS || (RW == 0 && G == 1), "block-wise compensation takes radius and stride at run time");
     static_assert(G == 1 || (!KAHAN && FMT == 0), "lane groups run the plain FP32 form");
@@ -1173,19 +1173,26 @@ __host__ __device__ constexpr int min_blocks(int prec, int th, int g) {
     return prec_blocks(prec) ? 3 : (prec & PREC_KAHAN) ? 1 : PC_MIN_BLOCKS * (8 / (th * g));
 }
 
+// Forms of the per-frame kernel: 32-pixel columns only; columns and strips;
+// the same with room for twice the registers a thread.  One warp alone on its
+// scheduler waits for its own results most of the time, and more of a window's
+// pairs in flight, which needs the registers, shorten those waits.
+enum Form { COLUMNS, STRIPS, ROOMY };
+
 // One CTA per tile of the band of pixel rows row0 .. row1 - 1 of the frame.
-template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS>
-__global__ void __launch_bounds__(cta_threads(PREC, TH, G), min_blocks(PREC, TH, G))
+template <int RW, bool REJECT, int PREC, int TH, int G, int RS, Form FORM>
+__global__ void __launch_bounds__(cta_threads(PREC, TH, G), FORM == ROOMY ? 8 / TH : min_blocks(PREC, TH, G))
     k_fit(FrameArgs f, FitConfig cfg, int row0, int row1) {
     extern __shared__ float smem[];
-    if constexpr (STRIPS) {
+    constexpr int AHEAD_FROM = FORM == ROOMY ? PC_AHEAD_BATCH : PC_AHEAD_FRAME;
+    if constexpr (FORM != COLUMNS) {
         const TilePos p = tile_pos(tiling_of(row1 - row0, f.W, TH, true), blockIdx.x, TH);
-        fit_tile<RW, REJECT, PREC, TH, G, RS, true, false>(f, cfg, p.ub, row0 + p.vb, p.lg, row1, smem);
+        fit_tile<RW, REJECT, PREC, TH, G, RS, true, AHEAD_FROM>(f, cfg, p.ub, row0 + p.vb, p.lg, row1, smem);
     } else {
         // a two-dimensional grid, so that nothing but the block and thread index
         // says where a pixel lies
-        fit_tile<RW, REJECT, PREC, TH, G, RS, false, false>(f, cfg, blockIdx.x * TILE_W, row0 + blockIdx.y * TH, 5, row1,
-                                                            smem);
+        fit_tile<RW, REJECT, PREC, TH, G, RS, false, AHEAD_FROM>(f, cfg, blockIdx.x * TILE_W, row0 + blockIdx.y * TH, 5,
+                                                                 row1, smem);
     }
 }
 
@@ -1212,7 +1219,7 @@ __global__ void __launch_bounds__(cta_threads(PREC, TH, G), min_blocks(PREC, TH,
         }
         const int H = fr[lo].f.H;
         const TilePos p = tile_pos(tiling_of(H, fr[lo].f.W, TH, G == 1), t - fr[lo].tile_begin, TH);
-        fit_tile<RW, REJECT, PREC, TH, G, RS, G == 1, true>(fr[lo].f, cfg, p.ub, p.vb, p.lg, H, smem);
+        fit_tile<RW, REJECT, PREC, TH, G, RS, G == 1, PC_AHEAD_BATCH>(fr[lo].f, cfg, p.ub, p.vb, p.lg, H, smem);
         __syncthreads();  // shared memory and s_tile are reused by the next tile
         if (threadIdx.x == 0 && threadIdx.y == 0) s_tile = (int)(gridDim.x + atomicAdd(next_tile, 1u));
         __syncthreads();
@@ -1250,17 +1257,28 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
         kernel<<<grid, block, smem, stream>>>(f, cfg, row0, row1);
         return cudaGetLastError();
     };
+    // A frame of at most one 128-thread CTA per SM (one warp per scheduler) takes
+    // the roomy form, which the SM could hold two of.  GB300, 160 x 120 / 109 x
+    // 82, T = 5, against 128 registers: r = 3 15.2 -> 14.3 / 15.9 -> 14.4 us, r =
+    // 7 57.4 -> 49.1 / 57.5 -> 49.4, r = 12 141 -> 116 / 141 -> 115, the 37 x 37
+    // patch 1.08 / 1.19 times as fast.  Radii 1 and 4 and the run-time kernels are
+    // level with it (0.96 to 1.05), and two CTAs per SM are no faster than one
+    // 32 x 8 tile.
+    if constexpr (PREC == 0 && G == 1 && TH == 4 && (RW / RS >= 5 || RW / RS == 3)) {
+        if (!cfg.reject && (int)strips.x <= cfg.sms) return launch(k_fit<RW, false, PREC, TH, G, RS, ROOMY>, strips);
+    }
     // Plain FP32 windows of 5 to 7 samples' radius without strips keep the form
     // that knows the tile's shape when compiled, whose loop needs no more
     // registers than it has (GB300, 640 x 480 frames alone: r = 6 3.577 against
     // 3.640 ms for eight, the 37 x 37 patch 3.622 against 3.690, r = 7 4.621
     // against 4.638); elsewhere the form with strips is as fast or faster.
     if constexpr (PREC == 0 && G == 1 && RW / RS >= 5 && RW / RS <= 7) {
-        if (!cfg.reject && tl.n16 + tl.n8 == 0) return launch(k_fit<RW, false, PREC, TH, G, RS, false>, columns);
+        if (!cfg.reject && tl.n16 + tl.n8 == 0) return launch(k_fit<RW, false, PREC, TH, G, RS, COLUMNS>, columns);
     }
+    constexpr Form FORM = G == 1 ? STRIPS : COLUMNS;
     const dim3 grid = G == 1 ? strips : columns;
-    return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, G == 1>, grid)
-                      : launch(k_fit<RW, false, PREC, TH, G, RS, G == 1>, grid);
+    return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, FORM>, grid)
+                      : launch(k_fit<RW, false, PREC, TH, G, RS, FORM>, grid);
 }
 
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>

@@ -31,6 +31,7 @@ struct FitConfig {
     int min_window;
     int kahan;         // compensated moment sums
     float fp64_pivot;  // refactorise in FP64 below this scaled pivot (0 = never)
+    int sms;           // SMs of the device launches go to (0: not known yet)
 };
 
 // Output tile of one CTA: TILE_W x th pixels, in five variants

@@ -167,8 +167,8 @@ pc_status pc_pack_depth(pc_ctx* ctx, const float* depth, int H, int W, int forma
 /* pc_compute reading the packed storage of pc_pack_depth (range = base +
  * offset, in FP32).  The arithmetic after loading is that of pc_compute; the
  * storage rounding is the only difference (its error against the FP64 oracle
- * is measured, not bounded by the FP32 tolerance).  Windows of radius 3, 7
- * and 11 (dense, plain sums) run kernels with unrolled columns, others the
+ * is measured, not bounded by the FP32 tolerance).  Dense windows of
+ * radius 1 to 12 (plain sums) run kernels with unrolled columns, others the
  * run-time-radius kernels; both give the same bits. */
 pc_status pc_compute_packed(pc_ctx* ctx, const unsigned short* packed, const float* tile_base,
                             int format, int H, int W, void* stream, float* k1_out, float* k2_out,
@@ -232,7 +232,7 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
  * start-up), and latency-bound loops cannot afford cudaMalloc, which can wait
  * for the whole device.  This entry point allocates nothing: its scratch (the
  * tile counter and a frame table of at most PC_STATIC_MAX_FRAMES frames) is a
- * fixed array inside the library (about 19 KB, held on every GPU that loads
+ * fixed array inside the library (about 25 KB, held on every GPU that loads
  * the library until the process exits), and the frame table is staged
  * through a fixed host array.  The paper has no counterpart.  It runs the
  * kernel variant pc_compute_batch runs with the same ctx (the lane group that

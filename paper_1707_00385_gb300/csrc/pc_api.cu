@@ -283,24 +283,22 @@ struct OpsTable {
 }  // namespace
 
 // Kernels of compensated sums.
-static const KernelOps* kahan_ops(const FitConfig& cfg, int format) {
-    return cfg.r / cfg.stride >= COMP_MIN_RADIUS ? ops_compensated(format) : ops_precision(1, format);
+static const KernelOps* kahan_ops(const FitConfig& cfg, bool packed) {
+    return cfg.r / cfg.stride >= COMP_MIN_RADIUS ? ops_compensated(packed) : ops_kahan(packed);
 }
 
 const KernelOps* select_ops(const FitConfig& cfg) {
-    if (cfg.kahan) return kahan_ops(cfg, 0);
+    if (cfg.kahan) return kahan_ops(cfg, false);
     static const OpsTable table;  // built once (thread-safe initialisation)
     const bool dense = cfg.stride == 1 && cfg.r >= 1 && cfg.r <= 12;
     if (cfg.r == SPARSE_RADIUS && cfg.stride == SPARSE_STRIDE) return &table.ops[13];
     return &table.ops[dense ? cfg.r : 0];
 }
 
-const KernelOps* select_packed_ops(const FitConfig& cfg, int format) {
-    if (!cfg.kahan && cfg.stride == 1) {
-        const KernelOps* k = format == 1 ? ops_packed_f16(cfg.r) : format == 2 ? ops_packed_bf16(cfg.r) : nullptr;
-        if (k) return k;
-    }
-    return cfg.kahan ? kahan_ops(cfg, format) : ops_precision(0, format);
+const KernelOps* select_packed_ops(const FitConfig& cfg) {
+    if (cfg.kahan) return kahan_ops(cfg, true);
+    const int r = cfg.stride == 1 && cfg.r <= 12 ? cfg.r : 0;
+    return r <= 6 ? ops_packed_r0_6(r) : ops_packed_r7_12(r);
 }
 
 const FitConfig& ctx_config(const pc_ctx* ctx) { return ctx->cfg; }
@@ -467,7 +465,7 @@ pc_status pc_compute(pc_ctx* ctx, const float* depth, int H, int W, void* stream
     if (st != PC_OK) return st;
     if (H == 0 || W == 0) return PC_OK;
     if ((st = check_buffers(depth, k1_out, k2_out, normal_out)) != PC_OK) return st;
-    const pcurv::FrameArgs f{depth, H, W, ctx->cam, k1_out, k2_out, normal_out, nullptr, nullptr};
+    const pcurv::FrameArgs f{depth, H, W, ctx->cam, k1_out, k2_out, normal_out, nullptr, nullptr, 0};
     const pcurv::KernelOps* ops = pcurv::select_ops(ctx->cfg);
     int v = 0;
     cudaError_t e = variant_for(ctx, ops, H, W, &v);
@@ -485,7 +483,7 @@ pc_status pc_autotune(pc_ctx* ctx, const float* depth, int H, int W, void* strea
     if (st != PC_OK) return st;
     if (H == 0 || W == 0) return PC_OK;
     if ((st = check_buffers(depth, k1_out, k2_out, normal_out)) != PC_OK) return st;
-    const pcurv::FrameArgs f{depth, H, W, ctx->cam, k1_out, k2_out, normal_out, nullptr, nullptr};
+    const pcurv::FrameArgs f{depth, H, W, ctx->cam, k1_out, k2_out, normal_out, nullptr, nullptr, 0};
     const pcurv::KernelOps* ops = pcurv::select_ops(ctx->cfg);
     cudaStream_t s = (cudaStream_t)stream;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -609,9 +607,9 @@ pc_status pc_compute_packed(pc_ctx* ctx, const unsigned short* packed, const flo
     if (!k1_out || !k2_out || !aligned4(k1_out) || !aligned4(k2_out) || !aligned4(normal_out) ||
         !is_device_ptr(k1_out) || !is_device_ptr(k2_out) || (normal_out && !is_device_ptr(normal_out)))
         return PC_ERR_INVALID_ARG;
-    const pcurv::FrameArgs f{nullptr, H, W, ctx->cam, k1_out, k2_out, normal_out, packed, tile_base};
+    const pcurv::FrameArgs f{nullptr, H, W, ctx->cam, k1_out, k2_out, normal_out, packed, tile_base, format};
     const cudaError_t e =
-        fit_frame(pcurv::select_packed_ops(ctx->cfg, format), 0, f, ctx->cfg, (cudaStream_t)stream);
+        fit_frame(pcurv::select_packed_ops(ctx->cfg), 0, f, ctx->cfg, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "pc_compute_packed launch");
     return PC_OK;
 }
@@ -660,7 +658,7 @@ pc_status pc_compute_host(pc_ctx* ctx, const float* depth_host, int H, int W, vo
     }
     cudaStream_t s = (cudaStream_t)stream;
     const pcurv::FrameArgs f{ctx->d_depth, H, W, ctx->cam, ctx->d_k1, ctx->d_k2,
-                             normal_host ? ctx->d_normal : nullptr, nullptr, nullptr};
+                             normal_host ? ctx->d_normal : nullptr, nullptr, nullptr, 0};
     const pcurv::KernelOps* ops = pcurv::select_ops(ctx->cfg);
     int v = 0;
     if ((e = variant_for(ctx, ops, H, W, &v)) != cudaSuccess) return cuda_fail(ctx, e, "pc_compute_host plan");
@@ -863,7 +861,7 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
         pcurv::BatchFrame& d = t->frames[k++];
         d.f = pcurv::FrameArgs{fr.depth, fr.H, fr.W,
                                pcurv::Camera{fr.fx, fr.fy, fr.cx, fr.cy, 1.f / fr.fx, 1.f / fr.fy},
-                               fr.k1, fr.k2, fr.normal, nullptr, nullptr};
+                               fr.k1, fr.k2, fr.normal, nullptr, nullptr, 0};
         d.tile_begin = begin;
         begin += (int)pcurv::tiles_of(fr.H, fr.W, v);
     }
@@ -926,7 +924,7 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
     BatchScratch& b = ctx->batch;
     pc_status st = ensure_batch(ctx, b, live);
     if (st != PC_OK) return st;
-    const pcurv::KernelOps* ops = pcurv::select_packed_ops(ctx->cfg, format);
+    const pcurv::KernelOps* ops = pcurv::select_packed_ops(ctx->cfg);
     cudaError_t e;
     if (b.packed_ops != ops) {  // sized once per kernel and device (ensure_batch resets it)
         int sms = 0, per_sm = 0;
@@ -951,7 +949,7 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
         pcurv::BatchFrame& d = t->frames[k++];
         d.f = pcurv::FrameArgs{nullptr, fr.H, fr.W,
                                pcurv::Camera{fr.fx, fr.fy, fr.cx, fr.cy, 1.f / fr.fx, 1.f / fr.fy},
-                               fr.k1, fr.k2, fr.normal, fr.packed, fr.tile_base};
+                               fr.k1, fr.k2, fr.normal, fr.packed, fr.tile_base, format};
         d.tile_begin = begin;
         begin += (int)pcurv::tiles_of(fr.H, fr.W, 0);
     }

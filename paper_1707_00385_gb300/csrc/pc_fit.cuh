@@ -146,13 +146,13 @@ __device__ __forceinline__ void local_xyz2(const Coef2& k, f32x2 Z, f32x2 DU, f3
     Hh = fma2(fma2(DU, k.cx2, RH), Z, mul2(k.bh, dZ));
 }
 
-// Precision variants of the kernels (template parameter PREC): bit 0 selects
-// compensated sums with every term compensated, bits 1-2 the range storage (0
-// float32, 1 FP16 offsets, 2 BF16 offsets from a per-tile base), bit 3 (with
-// bit 0) compensated sums of which J^T W J is compensated column block by
-// column block (fold_compensated).
-constexpr int PREC_KAHAN = 1, PREC_BLOCKS = 8;
-__host__ __device__ constexpr int prec_format(int prec) { return (prec >> 1) & 3; }
+// Precision variants of the kernels (template parameter PREC): compensated sums
+// with every term compensated, or of which J^T W J is compensated column block
+// by column block (fold_compensated); and ranges read from 16-bit storage,
+// whose format FrameArgs tells (the load is a few instructions of a tile's
+// staging, so one instantiation reads both formats).
+constexpr int PREC_KAHAN = 1, PREC_BLOCKS = 2, PREC_PACKED = 4;
+__host__ __device__ constexpr bool prec_kahan(int prec) { return (prec & PREC_KAHAN) != 0; }
 __host__ __device__ constexpr bool prec_blocks(int prec) { return (prec & PREC_BLOCKS) != 0; }
 // Threads of a CTA: one per pixel and lane, half of that in the block-wise
 // compensated form, whose threads take two pixels one after the other.
@@ -834,18 +834,18 @@ __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_r
 template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS, int AHEAD_FROM>
 __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cfg, int ub, int vb, int lg, int vend,
                                          float* smem) {
-    constexpr bool BLOCKS = prec_blocks(PREC);                   // J^T W J compensated block by block
-    constexpr bool KAHAN = (PREC & PREC_KAHAN) != 0 && !BLOCKS;  // every term compensated
-    constexpr int FMT = prec_format(PREC);
+    constexpr bool KAHAN = prec_kahan(PREC), BLOCKS = prec_blocks(PREC);
+    constexpr bool PACKED = (PREC & PREC_PACKED) != 0;
     constexpr int NT = cta_threads(PREC, TH, G), NW = NT / 32;   // threads and warps of the CTA
     constexpr int PARTS = TILE_W * TH * G / NT;                  // pixels of a thread, one after the other
     // fold the J^T W J sums row by row (one thread per pixel, plain sums)
     constexpr bool FOLD = G == 1 && !KAHAN && !BLOCKS;
-    // form each pair's state one pair ahead
-    constexpr bool AHEAD = FOLD && RW / RS >= AHEAD_FROM;
+    // form each pair's state one pair ahead (with rejection it is level or, from
+    // radius 11, slower: 927 x 486, r = 12 3.699 against 3.618 ms)
+    constexpr bool AHEAD = FOLD && !REJECT && RW / RS >= AHEAD_FROM;
     static_assert(G == 1 || G == 2 || G == 4 || G == 8, "lanes per pixel");
     static_assert(!BLOCKS || (RW == 0 && G == 1), "block-wise compensation takes radius and stride at run time");
-    static_assert(G == 1 || (!KAHAN && FMT == 0), "lane groups run the plain FP32 form");
+    static_assert(G == 1 || PREC == 0, "lane groups run the plain FP32 form");
     static_assert(G == 1 || RW == 0 || RS == 1, "lane groups with a compile-time window are dense");
     const float* __restrict__ depth = f.depth;
     const int H = f.H, W = f.W;
@@ -894,12 +894,12 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
             float z = 0.f, c = __int_as_float(0x7f800000);
             if (sx < SWU && row_in && gu >= 0 && gu < W) {
                 float d;
-                if (FMT == 0) {
+                if (!PACKED) {
                     d = __ldg(depth + (size_t)gv * W + gu);
                 } else {
                     // centred 16-bit storage: range = tile base + offset
                     const unsigned short q = __ldg(f.packed + (size_t)gv * W + gu);
-                    const float off = FMT == 1 ? __half2float(__ushort_as_half(q))
+                    const float off = f.format == 1 ? __half2float(__ushort_as_half(q))
                                                : __bfloat162float(__ushort_as_bfloat16(q));
                     d = __ldg(f.tile_base + (size_t)(gv / PACK_TILE_H) * ((W + TILE_W - 1) / TILE_W) +
                               gu / TILE_W) +
@@ -1030,8 +1030,10 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         // The window's row addresses are the same in every iteration.  Made opaque
         // here, they are computed again instead of all being kept in registers,
         // which spilled for small windows (GB300, 640 x 480, T = 5, a frame
-        // batched: r = 2 94.3 -> 88.4 us, r = 14 2.404 -> 2.314 ms alone).
-        if (STRIPS) asm volatile("" : "+r"(SW));
+        // batched: r = 2 94.3 -> 88.4 us, r = 14 2.404 -> 2.314 ms alone).  Not in
+        // the run-time loops with rejection: there it cost small frames 9 % (64 x
+        // 49, r = 14: 328 -> 357 us).
+        if (STRIPS && !(RW == 0 && REJECT)) asm volatile("" : "+r"(SW));
         const float *zc = tz + cidx, *cc = tcv + cidx;
         Moments2 m, comp;
         zero(m);
@@ -1170,7 +1172,7 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
 // threads (168 registers: the compensations of the eps sums; GB300, 640 x 480,
 // r = 7: 0.985 ms a frame against 1.034 with four at 128 registers).
 __host__ __device__ constexpr int min_blocks(int prec, int th, int g) {
-    return prec_blocks(prec) ? 3 : (prec & PREC_KAHAN) ? 1 : PC_MIN_BLOCKS * (8 / (th * g));
+    return prec_blocks(prec) ? 3 : prec_kahan(prec) ? 1 : PC_MIN_BLOCKS * (8 / (th * g));
 }
 
 // Forms of the per-frame kernel: 32-pixel columns only; columns and strips;
@@ -1231,7 +1233,7 @@ __global__ void __launch_bounds__(cta_threads(PREC, TH, G), min_blocks(PREC, TH,
 // one-thread FP32 kernels, the folded totals of its 32 x TH threads.
 template <int PREC, int TH, int G>
 size_t variant_smem_bytes(const FitConfig& cfg) {
-    constexpr bool TOTALS = G == 1 && ((PREC & PREC_KAHAN) == 0 || prec_blocks(PREC));
+    constexpr bool TOTALS = G == 1 && !prec_kahan(PREC);
     return fit_smem_bytes(cfg, TH, G == 1, TOTALS ? cta_threads(PREC, TH, G) : 0);
 }
 
@@ -1267,13 +1269,15 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
     if constexpr (PREC == 0 && G == 1 && TH == 4 && (RW / RS >= 5 || RW / RS == 3)) {
         if (!cfg.reject && (int)strips.x <= cfg.sms) return launch(k_fit<RW, false, PREC, TH, G, RS, ROOMY>, strips);
     }
-    // Plain FP32 windows of 5 to 7 samples' radius without strips keep the form
-    // that knows the tile's shape when compiled, whose loop needs no more
-    // registers than it has (GB300, 640 x 480 frames alone: r = 6 3.577 against
-    // 3.640 ms for eight, the 37 x 37 patch 3.622 against 3.690, r = 7 4.621
-    // against 4.638); elsewhere the form with strips is as fast or faster.
-    if constexpr (PREC == 0 && G == 1 && RW / RS >= 5 && RW / RS <= 7) {
-        if (!cfg.reject && tl.n16 + tl.n8 == 0) return launch(k_fit<RW, false, PREC, TH, G, RS, COLUMNS>, columns);
+    // Plain sums over windows of 5 to 7 samples' radius keep, where there are no
+    // strips, the form that knows the tile's shape when compiled, whose loop needs
+    // no more registers than it has (GB300, 640 x 480 frames alone: r = 6 3.577
+    // against 3.640 ms for eight, the 37 x 37 patch 3.622 against 3.690, r = 7
+    // 4.621 against 4.638); elsewhere the form with strips is as fast or faster.
+    if constexpr ((PREC & ~PREC_PACKED) == 0 && G == 1 && RW / RS >= 5 && RW / RS <= 7) {
+        if (tl.n16 + tl.n8 == 0)
+            return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, COLUMNS>, columns)
+                              : launch(k_fit<RW, false, PREC, TH, G, RS, COLUMNS>, columns);
     }
     constexpr Form FORM = G == 1 ? STRIPS : COLUMNS;
     const dim3 grid = G == 1 ? strips : columns;
@@ -1319,6 +1323,15 @@ const KernelOps* make_ops() {
     static const KernelOps k = {{launch_fit_rw<RW, PREC, 8, 1, RS>, launch_fit_rw<RW, PREC, 4, 1, RS>},
                                 {launch_batch_rw<RW, PREC, 8, 1, RS>, launch_batch_rw<RW, PREC, 4, 1, RS>},
                                 {occupancy_rw<RW, PREC, 8, 1, RS>, occupancy_rw<RW, PREC, 4, 1, RS>}};
+    return &k;
+}
+
+// The 32 x 8 one-lane variant alone.
+template <int RW, int PREC>
+const KernelOps* make_ops8() {
+    static const KernelOps k = {{launch_fit_rw<RW, PREC, 8>, nullptr},
+                                {launch_batch_rw<RW, PREC, 8>, nullptr},
+                                {occupancy_rw<RW, PREC, 8>, nullptr}};
     return &k;
 }
 

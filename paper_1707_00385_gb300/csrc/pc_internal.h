@@ -144,10 +144,11 @@ struct FrameArgs {
     float* k1;
     float* k2;
     float* normal;  // may be nullptr
-    // centred 16-bit storage instead of depth (precision variants): per pixel
-    // an offset, per 32x8 tile an FP32 base
+    // centred 16-bit storage instead of depth (the kernels reading it): per
+    // pixel an offset (format 1 FP16, 2 BF16), per 32x8 tile an FP32 base
     const unsigned short* packed;
     const float* tile_base;
+    int format;
 };
 
 // A frame of a batch and its place in the flattened tile queue.
@@ -192,12 +193,11 @@ const KernelOps* ops_lanes();
 constexpr int SPARSE_RADIUS = 18, SPARSE_STRIDE = 3;
 const KernelOps* ops_sparse(int r, int stride);
 
-// Run-time-radius kernels of the precision variants: compensated sums and/or
-// 16-bit range storage (format 0 float32, 1 FP16, 2 BF16).
-const KernelOps* ops_precision(int kahan, int format);
-// The block-wise compensated form of the same (kernels of compensated sums from
-// COMP_MIN_RADIUS samples to each side), else nullptr.
-const KernelOps* ops_compensated(int format);
+// Kernels of compensated sums (run-time radius and stride), for float32 ranges
+// or 16-bit storage: every term compensated, and J^T W J block by block (from
+// COMP_MIN_RADIUS samples to each side).
+const KernelOps* ops_kahan(bool packed);
+const KernelOps* ops_compensated(bool packed);
 // Window radius (in samples) from which J^T W J is compensated block by block.
 // GB300, one 640 x 480 frame alone, T = 5, every term / block-wise: r = 5 0.950
 // / 0.582 ms, r = 7 1.707 / 0.984, r = 12 4.608 / 2.702.  Against 64 bits the
@@ -208,12 +208,13 @@ const KernelOps* ops_compensated(int format);
 // 0.9538 / 0.9561).  At r = 3, whose blocks are a third of the window, 0.9904 /
 // 0.9899: smaller windows keep every term compensated.
 constexpr int COMP_MIN_RADIUS = 5;
-// 16-bit range storage with unrolled columns for window radii 3, 7 and 11
-// (plain sums), else nullptr.
-const KernelOps* ops_packed_f16(int r);
-const KernelOps* ops_packed_bf16(int r);
-// The kernels reading 16-bit storage of `format` (1 FP16, 2 BF16) under cfg.
-const KernelOps* select_packed_ops(const FitConfig& cfg, int format);
+// Plain sums on 16-bit range storage, 32 x 8 tiles: dense windows of radius 1
+// to 6 and 7 to 12 with unrolled columns (nullptr outside), and run-time radius
+// and stride (r = 0).
+const KernelOps* ops_packed_r0_6(int r);
+const KernelOps* ops_packed_r7_12(int r);
+// The kernels reading 16-bit storage (either format) under cfg.
+const KernelOps* select_packed_ops(const FitConfig& cfg);
 
 // The instantiation serving cfg (dense radii 1..12 unrolled, anything else
 // run-time; compensated sums on the precision kernels), all five variants.

@@ -145,7 +145,7 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
         pcurv::BatchFrame& d = t->frames[k++];
         d.f = pcurv::FrameArgs{f.depth, f.H, f.W,
                                pcurv::Camera{f.fx, f.fy, f.cx, f.cy, 1.f / f.fx, 1.f / f.fy},
-                               f.k1, f.k2, f.normal, nullptr, nullptr};
+                               f.k1, f.k2, f.normal, nullptr, nullptr, 0};
         d.tile_begin = begin;
         begin += (int)pcurv::tiles_of(f.H, f.W, v);
     }

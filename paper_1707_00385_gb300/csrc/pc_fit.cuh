@@ -1030,10 +1030,8 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         // The window's row addresses are the same in every iteration.  Made opaque
         // here, they are computed again instead of all being kept in registers,
         // which spilled for small windows (GB300, 640 x 480, T = 5, a frame
-        // batched: r = 2 94.3 -> 88.4 us, r = 14 2.404 -> 2.314 ms alone).  Not in
-        // the run-time loops with rejection: there it cost small frames 9 % (64 x
-        // 49, r = 14: 328 -> 357 us).
-        if (STRIPS && !(RW == 0 && REJECT)) asm volatile("" : "+r"(SW));
+        // batched: r = 2 94.3 -> 88.4 us, r = 14 2.404 -> 2.314 ms alone).
+        if (STRIPS) asm volatile("" : "+r"(SW));
         const float *zc = tz + cidx, *cc = tcv + cidx;
         Moments2 m, comp;
         zero(m);
@@ -1278,6 +1276,14 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
         if (tl.n16 + tl.n8 == 0)
             return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, COLUMNS>, columns)
                               : launch(k_fit<RW, false, PREC, TH, G, RS, COLUMNS>, columns);
+    }
+    // So do the run-time loops with rejection in frames of few tiles, ragged or
+    // not (64 x 49, T = 5: r = 14 328 us against 356 with the general form, r = 12
+    // sampled every 3 41.5 against 45.2; from 320 x 241 up the two are level).
+    if constexpr (PREC == 0 && G == 1 && RW == 0) {
+        const Tiling tc = tiling_of(row1 - row0, f.W, TH, false);
+        if (cfg.reject && (tl.n16 + tl.n8 == 0 || tc.full <= 2 * cfg.sms))
+            return launch(k_fit<RW, true, PREC, TH, G, RS, COLUMNS>, dim3(tc.cols, (row1 - row0 + TH - 1) / TH));
     }
     constexpr Form FORM = G == 1 ? STRIPS : COLUMNS;
     const dim3 grid = G == 1 ? strips : columns;

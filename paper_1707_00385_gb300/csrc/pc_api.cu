@@ -703,8 +703,7 @@ pc_status pc_compute_host(pc_ctx* ctx, const float* depth_host, int H, int W, vo
     int copied = 0;  // rows of ranges enqueued so far
     for (int b = 0; b < bands; b++) {
         const int ty0 = (int)((long long)rows * b / bands), ty1 = (int)((long long)rows * (b + 1) / bands);
-        const int last = ty1 * th + halo;
-        const int need = b + 1 < bands && last < H ? last : H;
+        const int need = b + 1 < bands ? pcurv::staged_end(ty1 * th, halo, H) : H;
         if (need > copied) {
             if ((e = cudaMemcpyAsync(ctx->d_depth + (size_t)copied * W, depth_host + (size_t)copied * W,
                                      (size_t)(need - copied) * W * sizeof(float), cudaMemcpyHostToDevice, p.in)) !=

@@ -882,9 +882,10 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         for (int k = 0; k <= 2 * r0; k += s) seg |= 1ull << k;
     }
     const int lane = threadIdx.x;
+    const int vread = staged_end(vend, halo, H);
     for (int sy = threadIdx.y; sy < SH; sy += NW) {
         const int gv = vb - halo + sy;
-        const bool row_in = gv >= 0 && gv < H;
+        const bool row_in = gv >= 0 && gv < vread;
         unsigned long long lo = 0, hi = 0;  // validity of columns 0..63, 64..95
 #pragma unroll
         for (int pass = 0; pass < 3; pass++) {

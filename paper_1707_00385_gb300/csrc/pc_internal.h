@@ -114,6 +114,13 @@ inline long long tiles_of(int rows, int W, int variant) {
     return (long long)t.full + t.n16 + t.n8;
 }
 
+// First row of the frame that a band ending at row vend does not read.  A strip
+// tile is taller than a tile row and may overhang the band; the band's windows
+// end `halo` rows past it, and the rows after those may not have been copied to
+// the device yet (pc_compute_host).  The staging stops here, and a band waits
+// for the copy of the rows up to here.
+PC_HD inline int staged_end(int vend, int halo, int H) { return H - vend > halo ? vend + halo : H; }
+
 // Row pitch of the staged planes of a tile tw pixels wide.  A warp of a strip
 // tile spans 2 rows of 16 or 4 rows of 8 pixels: the pitch is padded so that
 // those rows fall into different shared-memory banks.

@@ -117,7 +117,10 @@ def test_host_entry_matches_device_entry(gpu):
 
 
 @pytest.mark.parametrize("H,W,r,params", [(480, 640, 7, {}), (720, 1280, 7, {}), (480, 640, 7, {"lanes_per_pixel": 2}),
-                                          (2000, 160, 7, {}), (480, 640, 12, {}), (480, 640, 3, {"tile_height": 4})])
+                                          (2000, 160, 7, {}), (480, 640, 12, {}), (480, 640, 3, {"tile_height": 4}),
+                                          # ragged widths: strip tiles that overhang a band's end
+                                          (480, 1000, 7, {}), (1003, 517, 3, {}), (481, 645, 14, {}),
+                                          (720, 1270, 7, {"tile_height": 8}), (333, 657, 7, {"reject": 1})])
 def test_host_entry_in_bands_matches_device_entry(gpu, H, W, r, params):
     """Frames of several waves of CTAs go through pc_compute_host in bands of
     tile rows (copies overlapping the kernels): the same bits as pc_compute,

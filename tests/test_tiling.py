@@ -2,7 +2,9 @@
 csrc/pc_internal.h's own functions, compiled into a small program.  Every pixel
 of every band belongs to exactly one tile, no tile starts outside, there are
 never more tiles than 32-pixel columns make, the staged rows of a warp fall
-into different shared-memory banks, and the planes fit the size requested."""
+into different shared-memory banks, and the planes fit the size requested.  A
+band of a frame stages every row its windows read and none after them, which
+the host entry may still be copying in."""
 import os
 import shutil
 import subprocess
@@ -32,7 +34,36 @@ static int check(int rows, int W, int th, bool strips) {
         if (h != 1) return 4;
     return 0;
 }
+// Bands of tile rows of an H x W frame, as the host entry cuts them; the ranges up
+// to `halo` rows past a band are on the device when its tiles run.
+static int check_bands(int H, int W, int th, int halo, int bands) {
+    const int rows_t = (H + th - 1) / th;
+    for (int b = 0; b < bands; b++) {
+        const int row0 = rows_t * b / bands * th, end = rows_t * (b + 1) / bands * th, row1 = end < H ? end : H;
+        const int copied = row1 + halo < H ? row1 + halo : H;
+        const Tiling t = tiling_of(row1 - row0, W, th, true);
+        for (int i = 0; i < t.full + t.n16 + t.n8; i++) {
+            const TilePos p = tile_pos(t, i, th);
+            const int first = row0 + p.vb, last = first + ((32 * th) >> p.lg) - 1;  // the tile's rows, its overhang too
+            const int limit = staged_end(row1, halo, H);
+            const int staged = last + halo < limit ? last + halo : limit - 1;       // last row it reads
+            const int live = last < row1 ? last : row1 - 1;                         // last row it computes
+            if (staged >= copied) return 1;
+            if (staged < (live + halo < H ? live + halo : H - 1)) return 2;
+        }
+    }
+    return 0;
+}
 int main() {
+    const int frames[][2] = {{1000, 480}, {1270, 720}, {1912, 1080}, {517, 1003}, {645, 481}, {657, 333}, {640, 480}, {9, 77}};
+    for (auto [W, H] : frames)
+        for (int th : {8, 4})
+            for (int halo : {1, 3, 7, 14, 24})
+                for (int bands = 1; bands <= 8; bands++)
+                    if (int e = check_bands(H, W, th, halo, bands)) {
+                        printf("%d x %d, th %d, halo %d, %d bands: %d\n", W, H, th, halo, bands, e);
+                        return 1;
+                    }
     for (int th : {8, 4, 2, 1})
         for (int strips = 0; strips <= (th >= 4); strips++)
             for (int W = 1; W <= 130; W++)

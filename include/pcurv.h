@@ -87,12 +87,8 @@ typedef struct pc_params {
                             table capacity; 0 = enqueue the three steps directly.  A batch
                             with fewer tiles than the persistent grid is always enqueued
                             directly, with one CTA per tile. Default 1 */
-    int kahan;           /* 1 = compensated (Kahan) summation of the window moments in FP32.
-                            Windows of five samples and more to each side add J^T W J in
-                            blocks of up to eight columns, each added with compensation, and
-                            compensate every term of J^T W eps; smaller windows compensate
-                            every term of both.  Costs about 1.7x (smaller windows 2.5x) the
-                            time of plain sums. Default 0 */
+    int kahan;           /* 1 = compensated (Kahan) summation of the window moments in FP32;
+                            costs about 2.9x the time of plain sums. Default 0 */
     float fp64_solve_cond; /* > 0: when the scaled condition estimate of the re-weighted system
                             (1 / smallest scaled pivot) exceeds this value, the 6x6 system is
                             factorised again in FP64 and singularity is judged on the FP64

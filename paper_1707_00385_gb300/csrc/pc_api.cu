@@ -282,13 +282,8 @@ struct OpsTable {
 
 }  // namespace
 
-// Kernels of compensated sums.
-static const KernelOps* kahan_ops(const FitConfig& cfg, bool packed) {
-    return cfg.r / cfg.stride >= COMP_MIN_RADIUS ? ops_compensated(packed) : ops_kahan(packed);
-}
-
 const KernelOps* select_ops(const FitConfig& cfg) {
-    if (cfg.kahan) return kahan_ops(cfg, false);
+    if (cfg.kahan) return ops_kahan(false);
     static const OpsTable table;  // built once (thread-safe initialisation)
     const bool dense = cfg.stride == 1 && cfg.r >= 1 && cfg.r <= 12;
     if (cfg.r == SPARSE_RADIUS && cfg.stride == SPARSE_STRIDE) return &table.ops[13];
@@ -296,7 +291,7 @@ const KernelOps* select_ops(const FitConfig& cfg) {
 }
 
 const KernelOps* select_packed_ops(const FitConfig& cfg) {
-    if (cfg.kahan) return kahan_ops(cfg, true);
+    if (cfg.kahan) return ops_kahan(true);
     const int r = cfg.stride == 1 && cfg.r <= 12 ? cfg.r : 0;
     return r <= 6 ? ops_packed_r0_6(r) : ops_packed_r7_12(r);
 }

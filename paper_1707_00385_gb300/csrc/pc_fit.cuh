@@ -146,19 +146,11 @@ __device__ __forceinline__ void local_xyz2(const Coef2& k, f32x2 Z, f32x2 DU, f3
     Hh = fma2(fma2(DU, k.cx2, RH), Z, mul2(k.bh, dZ));
 }
 
-// Precision variants of the kernels (template parameter PREC): compensated sums
-// with every term compensated, or of which J^T W J is compensated column block
-// by column block (fold_compensated); and ranges read from 16-bit storage,
-// whose format FrameArgs tells (the load is a few instructions of a tile's
-// staging, so one instantiation reads both formats).
-constexpr int PREC_KAHAN = 1, PREC_BLOCKS = 2, PREC_PACKED = 4;
-__host__ __device__ constexpr bool prec_kahan(int prec) { return (prec & PREC_KAHAN) != 0; }
-__host__ __device__ constexpr bool prec_blocks(int prec) { return (prec & PREC_BLOCKS) != 0; }
-// Threads of a CTA: one per pixel and lane, half of that in the block-wise
-// compensated form, whose threads take two pixels one after the other.
-__host__ __device__ constexpr int cta_threads(int prec, int th, int g) {
-    return TILE_W * th * g / (prec_blocks(prec) ? 2 : 1);
-}
+// Precision variants of the kernels (template parameter PREC): compensated sums;
+// and ranges read from 16-bit storage, whose format FrameArgs tells (the load is
+// a few instructions of a tile's staging, so one instantiation reads both
+// formats).
+constexpr int PREC_KAHAN = 1, PREC_PACKED = 2;
 
 // sum += a * b, plain or compensated.  The compensated form (Kahan) keeps
 // nc = -(rounding error so far): y = a b - c, t = s + y, c' = (t - s) - y.
@@ -228,9 +220,8 @@ __device__ __forceinline__ PairState pair_state(const Coef2& k, float za, float 
 }
 
 // The 26 sums of a pair (the eps sums scaled by sigma).  c holds the
-// compensations of the sums when KAHAN, those of the six eps sums alone when
-// only KAHAN_EPS (unused otherwise).
-template <bool KAHAN, bool FIRST, bool KAHAN_EPS = KAHAN>
+// compensations of the sums when KAHAN (unused otherwise).
+template <bool KAHAN, bool FIRST>
 __device__ __forceinline__ void add_pair(Moments2& m, Moments2& c, const PairState& p) {
     const f32x2 XX = mul2(p.X, p.X), XY = mul2(p.X, p.Y), YY = mul2(p.Y, p.Y);
     const f32x2 WE = mul2(p.Wt, p.E), WJ0 = mul2(p.Wt, p.NJ0), WJ1 = mul2(p.Wt, p.J1);
@@ -243,7 +234,7 @@ __device__ __forceinline__ void add_pair(Moments2& m, Moments2& c, const PairSta
     acc_add<KAHAN>(m.sw, c.sw, p.Wt);
     acc_add<KAHAN>(m.sxx, c.sxx, WXX);
     acc_add<KAHAN>(m.syy, c.syy, WYY);
-    acc_add<KAHAN_EPS>(m.ge, c.ge, WE);
+    acc_add<KAHAN>(m.ge, c.ge, WE);
     if (!FIRST) {
         // with j1 = x, -j0 = y these are sum w y^2, w x y, w x^2, w x^2 y, w x y^2
         acc_fma<KAHAN>(m.h00, c.h00, WJ0, p.NJ0);
@@ -258,11 +249,11 @@ __device__ __forceinline__ void add_pair(Moments2& m, Moments2& c, const PairSta
     }
     acc_fma<KAHAN>(m.h13, c.h13, WJ1, XX);
     if (!FIRST) acc_fma<KAHAN>(m.h11, c.h11, WJ1, p.J1);
-    acc_fma<KAHAN_EPS>(m.g1, c.g1, WE, p.J1);
-    acc_fma<KAHAN_EPS>(m.g0, c.g0, WE, p.NJ0);
-    acc_fma<KAHAN_EPS>(m.g3, c.g3, WE, XX);
-    acc_fma<KAHAN_EPS>(m.g4, c.g4, WE, XY);
-    acc_fma<KAHAN_EPS>(m.g5, c.g5, WE, YY);
+    acc_fma<KAHAN>(m.g1, c.g1, WE, p.J1);
+    acc_fma<KAHAN>(m.g0, c.g0, WE, p.NJ0);
+    acc_fma<KAHAN>(m.g3, c.g3, WE, XX);
+    acc_fma<KAHAN>(m.g4, c.g4, WE, XY);
+    acc_fma<KAHAN>(m.g5, c.g5, WE, YY);
     acc_fma<KAHAN>(m.m04, c.m04, WYY, YY);
     acc_fma<KAHAN>(m.m13, c.m13, WYY, XY);
     acc_fma<KAHAN>(m.sxy, c.sxy, p.Wt, XY);
@@ -314,42 +305,6 @@ __device__ __forceinline__ void fold_rows(Moments2& m, f32x2* tot, int nt) {
 template <bool FIRST>
 __device__ __forceinline__ void fold_finish(Moments2& m, const f32x2* tot, int nt) {
 #define PC_FOLD_ONE(i, f) m.f = add2(m.f, tot[(i) * nt]);
-    PC_FOLD_FIRST(PC_FOLD_ONE)
-    if (!FIRST) { PC_FOLD_LATER(PC_FOLD_ONE) }
-#undef PC_FOLD_ONE
-}
-
-// Columns of a window row whose J^T W J terms are summed plainly between two
-// compensated additions, at most.
-constexpr int COMP_COLUMNS = 8;
-
-// The compensated form of the fold: each of the 20 totals is a (sum, lost
-// part) pair, to which the partial sum of up to COMP_COLUMNS pairs is added
-// with Kahan's compensation; partial = 0.  Compensating every term takes three
-// more operations for each of the 26 sums of every pair (133 packed operations
-// a pair instead of 55, and 52 more registers).  Here the six eps sums, whose
-// terms change sign and whose sum settles the solution, keep that, and the 20
-// sums of J^T W J take five scalar operations each every eight pairs.
-template <bool FIRST>
-__device__ __forceinline__ void fold_compensated(Moments2& m, float2* tot, int nt) {
-#define PC_FOLD_ONE(i, f) { \
-        float2 t = tot[(i) * nt]; \
-        const float y = hsum(m.f) + t.y, sum = t.x + y; \
-        tot[(i) * nt] = make_float2(sum, y - (sum - t.x)); \
-        m.f = 0ull; \
-    }
-    PC_FOLD_FIRST(PC_FOLD_ONE)
-    if (!FIRST) { PC_FOLD_LATER(PC_FOLD_ONE) }
-#undef PC_FOLD_ONE
-}
-
-// The 20 sums as (sum, lost part) pairs, whose halves the solve adds.
-template <bool FIRST>
-__device__ __forceinline__ void take_compensated(Moments2& m, const float2* tot, int nt) {
-#define PC_FOLD_ONE(i, f) { \
-        const float2 t = tot[(i) * nt]; \
-        m.f = pack(t.x, t.y); \
-    }
     PC_FOLD_FIRST(PC_FOLD_ONE)
     if (!FIRST) { PC_FOLD_LATER(PC_FOLD_ONE) }
 #undef PC_FOLD_ONE
@@ -436,19 +391,17 @@ __device__ __forceinline__ void ldlt6(const T (&H)[6][6], const T (&g)[6], T del
     low = under;
 }
 
-// Folds the 26 pairs (with their compensations when KAHAN; those of the eps
-// sums when KAHAN_EPS), adds the centre
+// Folds the 26 pairs (with their compensations when KAHAN), adds the centre
 // point (w_c to sum w, w_c eps_c to sum w eps), assembles J^T W J and J^T W eps
 // and solves for the update delta = -b.  Singular when a diagonal entry is
 // <= 0 or a scaled pivot is <= pivot_tol; with fp64_pivot > 0 a system whose
 // smallest FP32 scaled pivot is below fp64_pivot is factorised again in FP64
 // and judged on the FP64 pivots.
-template <bool KAHAN, bool KAHAN_EPS>
+template <bool KAHAN>
 __device__ __forceinline__ bool solve_update(const Moments2& m, const Moments2& c, float wc, float ec,
                                              float isig, float pivot_tol, float fp64_pivot,
                                              float delta[6]) {
 #define PC_FOLD(f) (KAHAN ? hsum(add2(m.f, c.f)) : hsum(m.f))
-#define PC_FOLD_EPS(f) (KAHAN_EPS ? hsum(add2(m.f, c.f)) : hsum(m.f))
     const float h00 = PC_FOLD(h00), h01 = -PC_FOLD(h01), h11 = PC_FOLD(h11);
     const float s0 = PC_FOLD(s0), s1 = PC_FOLD(s1);
     const float h03 = -PC_FOLD(h03), h04 = -PC_FOLD(h04), h05 = -PC_FOLD(h05);
@@ -458,11 +411,9 @@ __device__ __forceinline__ bool solve_update(const Moments2& m, const Moments2& 
     const float m40 = PC_FOLD(m40), m31 = PC_FOLD(m31), m22 = PC_FOLD(m22), m13 = PC_FOLD(m13),
                 m04 = PC_FOLD(m04);
     // the eps sums carry sigma = 1/sqrt(k): isig = sqrt(k) restores them
-    const float g0 = -PC_FOLD_EPS(g0) * isig, g1 = PC_FOLD_EPS(g1) * isig,
-                ge = fmaf(wc, ec, PC_FOLD_EPS(ge) * isig);
-    const float g3 = PC_FOLD_EPS(g3) * isig, g4 = PC_FOLD_EPS(g4) * isig, g5 = PC_FOLD_EPS(g5) * isig;
+    const float g0 = -PC_FOLD(g0) * isig, g1 = PC_FOLD(g1) * isig, ge = fmaf(wc, ec, PC_FOLD(ge) * isig);
+    const float g3 = PC_FOLD(g3) * isig, g4 = PC_FOLD(g4) * isig, g5 = PC_FOLD(g5) * isig;
 #undef PC_FOLD
-#undef PC_FOLD_EPS
     float H[6][6];
     H[0][0] = h00; H[0][1] = h01; H[0][2] = s0;
     H[0][3] = 0.5f * h03; H[0][4] = h04; H[0][5] = 0.5f * h05;
@@ -634,38 +585,6 @@ __device__ __forceinline__ void for_each_pair_ahead(const float* zc, const float
     sums(p);
 }
 
-// for_each_pair at run-time radius and stride with the columns of each row in
-// blocks of equal length, at most COMP_COLUMNS; block_end() is called after
-// every block.
-template <typename F, typename E>
-__device__ __forceinline__ void for_each_pair_blocks(const float* zc, const float* cc, int SW, int r, int s, F&& f,
-                                                     E&& block_end) {
-    const f32x2 STEP = pack((float)s, -(float)s);
-    const int half = r / s, r0 = half * s;
-    const int columns = 2 * half + 1, blocks = (columns + COMP_COLUMNS - 1) / COMP_COLUMNS;
-    const int block = (columns + blocks - 1) / blocks;
-    for (int dv = -r0; dv <= 0; dv += s) {
-        const float *za = zc + dv * SW - r0, *zb = zc - dv * SW + r0;
-        const float *ca = cc + dv * SW - r0, *cb = cc - dv * SW + r0;
-        const f32x2 DV = pack((float)dv, -(float)dv);
-        f32x2 DU = pack(-(float)r0, (float)r0);
-        const int n = dv < 0 ? columns : half;  // the centre row's left half
-        for (int i = 0; i < n;) {
-            const int end = i + block < n ? i + block : n;
-#pragma unroll 2
-            for (; i < end; i++) {
-                f(*za, *zb, *ca, *cb, DU, DV);
-                za += s;
-                zb -= s;
-                ca += s;
-                cb -= s;
-                DU = add2(DU, STEP);
-            }
-            block_end();
-        }
-    }
-}
-
 // The share of one lane of a group of G lanes that computes one pixel
 // together: the window splits into row units, units 0 .. r0/s - 1 being the
 // rows dv = -r0 + k s (each point paired with its reflection (-du, -dv)) and
@@ -834,17 +753,14 @@ __device__ __forceinline__ bool initial_normal(const float* zc, int SW, int rn_r
 template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool STRIPS, int AHEAD_FROM>
 __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cfg, int ub, int vb, int lg, int vend,
                                          float* smem) {
-    constexpr bool KAHAN = prec_kahan(PREC), BLOCKS = prec_blocks(PREC);
-    constexpr bool PACKED = (PREC & PREC_PACKED) != 0;
-    constexpr int NT = cta_threads(PREC, TH, G), NW = NT / 32;   // threads and warps of the CTA
-    constexpr int PARTS = TILE_W * TH * G / NT;                  // pixels of a thread, one after the other
+    constexpr bool KAHAN = (PREC & PREC_KAHAN) != 0, PACKED = (PREC & PREC_PACKED) != 0;
+    constexpr int NW = TH * G;  // warps of the CTA
     // fold the J^T W J sums row by row (one thread per pixel, plain sums)
-    constexpr bool FOLD = G == 1 && !KAHAN && !BLOCKS;
+    constexpr bool FOLD = G == 1 && !KAHAN;
     // form each pair's state one pair ahead (with rejection it is level or, from
     // radius 11, slower: 927 x 486, r = 12 3.699 against 3.618 ms)
     constexpr bool AHEAD = FOLD && !REJECT && RW / RS >= AHEAD_FROM;
     static_assert(G == 1 || G == 2 || G == 4 || G == 8, "lanes per pixel");
-    static_assert(!BLOCKS || (RW == 0 && G == 1), "block-wise compensation takes radius and stride at run time");
     static_assert(G == 1 || PREC == 0, "lane groups run the plain FP32 form");
     static_assert(G == 1 || RW == 0 || RS == 1, "lane groups with a compile-time window are dense");
     const float* __restrict__ depth = f.depth;
@@ -868,7 +784,6 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
     int* rcnt = (int*)(tcv + SW * SH);      // valid window points per (tile row, pixel column)
     // folded totals: FOLD_SUMS pairs per thread after the planes (8-byte aligned)
     f32x2* fold_tot = (f32x2*)(smem + ((2 * SW * SH + SH * TW + 1) & ~1)) + tid;
-    float2* comp_tot = (float2*)fold_tot;   // block-wise compensation: (sum, lost part)
 
     // stage the tile + halo (Sec. 3.2, first item: the range image): warp w
     // takes halo rows w, w + NW, ..., its lanes the columns in passes of 32.
@@ -927,12 +842,11 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
     }
     __syncthreads();
 
-    auto pixel = [&](int part) {
     // the thread's pixel (tile column pxl, row pyl) and its lane in the group
     int pxl, pyl, sub = 0;
     if constexpr (G == 1 && STRIPS) {
-        pxl = (tid + part * NT) & (TW - 1);
-        pyl = (tid + part * NT) >> lg;
+        pxl = tid & (TW - 1);
+        pyl = tid >> lg;
     } else if constexpr (G == 1) {
         pxl = threadIdx.x;
         pyl = threadIdx.y;
@@ -1051,6 +965,7 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         };
         // fold the J^T W J partials after every PC_FOLD_ROWS pairs of rows: the
         // first fold starts the totals, the centre row's partial joins at the end
+        constexpr int NT = TILE_W * TH;
         const bool folded = FOLD && r0 / s >= 2 * PC_FOLD_ROWS;
         auto fold_first = [&](int row) {
             if constexpr (FOLD) {
@@ -1066,21 +981,9 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
                 else fold_rows<false>(m, fold_tot, NT);
             }
         };
-        if constexpr (BLOCKS) {
-#pragma unroll
-            for (int i = 0; i < FOLD_SUMS; i++) comp_tot[i * NT] = make_float2(0.f, 0.f);
-        }
         if (it == 0) {
             // A = B = C = 0 here: the cheaper first-iteration form
-            if constexpr (BLOCKS) {
-                for_each_pair_blocks(
-                    zc, cc, SW, r, s,
-                    [&](float za, float zb, float ca, float cb, f32x2 DU, f32x2 DV) {
-                        add_pair<false, true, true>(m, comp, state_first(za, zb, ca, cb, DU, DV));
-                    },
-                    [&]() { fold_compensated<true>(m, comp_tot, NT); });
-                take_compensated<true>(m, comp_tot, NT);
-            } else if constexpr (G == 1) {
+            if constexpr (G == 1) {
                 if constexpr (AHEAD)
                     for_each_pair_ahead<RW, RS>(
                         zc, cc, SW, state_first, [&](const PairState& p) { add_pair<false, true>(m, comp, p); }, fold_first);
@@ -1092,15 +995,7 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
             }
             first_iteration_sums(m, comp);
         } else {
-            if constexpr (BLOCKS) {
-                for_each_pair_blocks(
-                    zc, cc, SW, r, s,
-                    [&](float za, float zb, float ca, float cb, f32x2 DU, f32x2 DV) {
-                        add_pair<false, false, true>(m, comp, state_later(za, zb, ca, cb, DU, DV));
-                    },
-                    [&]() { fold_compensated<false>(m, comp_tot, NT); });
-                take_compensated<false>(m, comp_tot, NT);
-            } else if constexpr (G == 1) {
+            if constexpr (G == 1) {
                 if constexpr (AHEAD)
                     for_each_pair_ahead<RW, RS>(
                         zc, cc, SW, state_later, [&](const PairState& p) { add_pair<false, false>(m, comp, p); }, fold_later);
@@ -1114,7 +1009,7 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         if constexpr (G > 1) reduce_lanes<G>(m);
 
         float dl[6];
-        const bool solved = solve_update<KAHAN, KAHAN || BLOCKS>(m, comp, wcr, ec, isig, cfg.pivot_tol, cfg.fp64_pivot, dl);
+        const bool solved = solve_update<KAHAN>(m, comp, wcr, ec, isig, cfg.pivot_tol, cfg.fp64_pivot, dl);
         if constexpr (G == 1) {
             if (!solved) {
                 ok = false;
@@ -1156,23 +1051,12 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         nrmo[3 * out + 1] = R[7];
         nrmo[3 * out + 2] = R[8];
     }
-    };
-    if constexpr (PARTS == 1) {
-        pixel(0);
-    } else {
-#pragma unroll 1
-        for (int part = 0; part < PARTS; part++) pixel(part);
-    }
 }
 
-// CTAs per SM that the registers of a variant are bounded for.  One thread per
-// pixel and plain sums: two of 256 threads.  Every term compensated: one (a
-// pair of registers more per sum).  Block-wise compensation: three of 128
-// threads (168 registers: the compensations of the eps sums; GB300, 640 x 480,
-// r = 7: 0.985 ms a frame against 1.034 with four at 128 registers).
-__host__ __device__ constexpr int min_blocks(int prec, int th, int g) {
-    return prec_blocks(prec) ? 3 : prec_kahan(prec) ? 1 : PC_MIN_BLOCKS * (8 / (th * g));
-}
+// Compensated sums need a pair of registers more per sum: those variants keep
+// one CTA per SM instead of spilling.
+#define PC_BLOCKS_OF(PREC) (((PREC) & PREC_KAHAN) ? 1 : PC_MIN_BLOCKS)
+
 
 // Forms of the per-frame kernel: 32-pixel columns only; columns and strips;
 // the same with room for twice the registers a thread.  One warp alone on its
@@ -1182,7 +1066,7 @@ enum Form { COLUMNS, STRIPS, ROOMY };
 
 // One CTA per tile of the band of pixel rows row0 .. row1 - 1 of the frame.
 template <int RW, bool REJECT, int PREC, int TH, int G, int RS, Form FORM>
-__global__ void __launch_bounds__(cta_threads(PREC, TH, G), FORM == ROOMY ? 8 / TH : min_blocks(PREC, TH, G))
+__global__ void __launch_bounds__(TILE_W * TH * G, FORM == ROOMY ? 8 / TH : PC_BLOCKS_OF(PREC) * (8 / (TH * G)))
     k_fit(FrameArgs f, FitConfig cfg, int row0, int row1) {
     extern __shared__ float smem[];
     constexpr int AHEAD_FROM = FORM == ROOMY ? PC_AHEAD_BATCH : PC_AHEAD_FRAME;
@@ -1204,7 +1088,7 @@ __global__ void __launch_bounds__(cta_threads(PREC, TH, G), FORM == ROOMY ? 8 / 
 // one atomic each.  The header and descriptors live in device memory
 // (BatchTable); *next_tile must be 0 at launch.
 template <int RW, bool REJECT, int PREC, int TH, int G, int RS>
-__global__ void __launch_bounds__(cta_threads(PREC, TH, G), min_blocks(PREC, TH, G))
+__global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH * G)))
     k_fit_batch(const BatchTable* __restrict__ table, unsigned* __restrict__ next_tile, FitConfig cfg) {
     extern __shared__ float smem[];
     __shared__ int s_tile;
@@ -1232,8 +1116,8 @@ __global__ void __launch_bounds__(cta_threads(PREC, TH, G), min_blocks(PREC, TH,
 // one-thread FP32 kernels, the folded totals of its 32 x TH threads.
 template <int PREC, int TH, int G>
 size_t variant_smem_bytes(const FitConfig& cfg) {
-    constexpr bool TOTALS = G == 1 && !prec_kahan(PREC);
-    return fit_smem_bytes(cfg, TH, G == 1, TOTALS ? cta_threads(PREC, TH, G) : 0);
+    constexpr bool FOLD = G == 1 && (PREC & PREC_KAHAN) == 0;
+    return fit_smem_bytes(cfg, TH, G == 1, FOLD ? TILE_W * TH : 0);
 }
 
 // Kernels whose dynamic shared memory exceeds the default 48 KB opt in on the
@@ -1247,7 +1131,7 @@ cudaError_t allow_smem(K kernel, size_t smem) {
 // Tile rows ty0 .. ty1 - 1 of the frame (0 <= ty0 < ty1 <= its tile rows).
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>
 cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t stream, int ty0, int ty1) {
-    const dim3 block(TILE_W, cta_threads(PREC, TH, G) / TILE_W);
+    const dim3 block(TILE_W, TH * G);
     const int row0 = ty0 * TH, row1 = ty1 * TH < f.H ? ty1 * TH : f.H;
     const Tiling tl = tiling_of(row1 - row0, f.W, TH, G == 1);
     const dim3 strips(tl.full + tl.n16 + tl.n8), columns(tl.cols, (row1 - row0 + TH - 1) / TH);
@@ -1295,7 +1179,7 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>
 cudaError_t launch_batch_rw(const BatchTable* table, unsigned* next_tile, int grid, const FitConfig& cfg,
                             cudaStream_t stream) {
-    const dim3 block(TILE_W, cta_threads(PREC, TH, G) / TILE_W);
+    const dim3 block(TILE_W, TH * G);
     const size_t smem = variant_smem_bytes<PREC, TH, G>(cfg);
     cudaError_t e;
     if (cfg.reject) {
@@ -1315,11 +1199,11 @@ cudaError_t occupancy_rw(const FitConfig& cfg, int* blocks_per_sm) {
     if (cfg.reject) {
         if ((e = allow_smem(k_fit_batch<RW, true, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_fit_batch<RW, true, PREC, TH, G, RS>,
-                                                             cta_threads(PREC, TH, G), smem);
+                                                             TILE_W * TH * G, smem);
     }
     if ((e = allow_smem(k_fit_batch<RW, false, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_fit_batch<RW, false, PREC, TH, G, RS>,
-                                                         cta_threads(PREC, TH, G), smem);
+                                                         TILE_W * TH * G, smem);
 }
 
 // The one-lane variants (32 x 8 and 32 x 4 tiles) of radius RW sampled every

@@ -1,5 +1,5 @@
-// Instantiations of compensated sums with every term compensated (run-time
-// radius and stride, 32 x 8 tiles, per-frame and persistent batch kernels).
+// Instantiations of compensated sums (run-time radius and stride, 32 x 8 tiles,
+// per-frame and persistent batch kernels).
 #include "pc_fit.cuh"
 
 namespace pcurv {

@@ -201,20 +201,8 @@ constexpr int SPARSE_RADIUS = 18, SPARSE_STRIDE = 3;
 const KernelOps* ops_sparse(int r, int stride);
 
 // Kernels of compensated sums (run-time radius and stride), for float32 ranges
-// or 16-bit storage: every term compensated, and J^T W J block by block (from
-// COMP_MIN_RADIUS samples to each side).
+// or 16-bit storage.
 const KernelOps* ops_kahan(bool packed);
-const KernelOps* ops_compensated(bool packed);
-// Window radius (in samples) from which J^T W J is compensated block by block.
-// GB300, one 640 x 480 frame alone, T = 5, every term / block-wise: r = 5 0.950
-// / 0.582 ms, r = 7 1.707 / 0.984, r = 12 4.608 / 2.702.  Against 64 bits the
-// two are level from 5 up (eight smooth surfaces, block-wise over every term,
-// geometric mean: r = 5 k1 1.002 k2 1.006, r = 7 0.999 and 1.003, r = 12 1.002
-// and 1.000, single surfaces 0.92 to 1.15; six Kinect-like frames, k1 of the
-// pixels within tolerance: r = 5 0.9791 / 0.9790, r = 7 0.9675 / 0.9675, r = 12
-// 0.9538 / 0.9561).  At r = 3, whose blocks are a third of the window, 0.9904 /
-// 0.9899: smaller windows keep every term compensated.
-constexpr int COMP_MIN_RADIUS = 5;
 // Plain sums on 16-bit range storage, 32 x 8 tiles: dense windows of radius 1
 // to 6 and 7 to 12 with unrolled columns (nullptr outside), and run-time radius
 // and stride (r = 0).

@@ -88,33 +88,44 @@ __global__ void __launch_bounds__(BP_THREADS, BP_BLOCKS_PER_SM)
 // One CTA per 32 x (TH PPT) output tile: each thread computes PPT pixels of
 // its column, TH rows apart, so that one staging of the tile's Z plane plus a
 // halo of rn (0 where the range is not valid, as the full path stages it)
-// serves PPT times the arithmetic.  A warp's 32 pixels share their patch rows:
-// where none of those rows of the staged tile has a point without a range
-// (holes, one flag per row), the warp takes the unmasked sums of
-// initial_normal, 13 packed operations a pair of points against 14 and two
-// selects, with the same bits.  The kernel is bound by the issue of those
-// operations: GB300, 4096 x 4096 with a hole of 2 to 8 pixels' radius in each
-// 64 x 64 pixels: point cloud and normals together 465.8 -> 438.0 us; one
-// 2048 x 2048 normal field 110.7 -> 104.6 us, 640 x 480 12.5 -> 12.4 us.  Registers are bounded for four 256-thread
+// serves PPT times the arithmetic.  Registers are bounded for four 256-thread
 // CTAs per SM (the 7x7 patch, unrolled, would otherwise take more and leave
 // three).
-template <int TH, int PPT>
+//
+// RN > 0: the patch radius, unrolled; RN = 0: radius rn_rt.  The unrolled 7x7
+// patch is bound by the issue of its packed operations.  A warp's 32 pixels
+// share their patch rows: where none of those rows of the staged tile has a
+// point without a range (holes, one flag per row), the warp takes the unmasked
+// sums of initial_normal, 13 packed operations a pair of points against 14 and
+// two selects, with the same bits.  One lane per pixel row looks at that row's
+// flags, once a tile, so that an image whose holes lie everywhere pays next to
+// nothing for them (looked at by every thread for every pixel, and in the
+// kernel of all radii, they cost such an image 3 % and the other radii up to
+// 6 %).  GB300, 4096 x 4096, normals alone, masked sums only / this kernel: no
+// hole 416.8 / 361.0 us, a disk of 5 pixels' radius in each 64 x 64 pixels
+// 417.1 / 368.1, single pixels, 0.1 % 417.3 / 375.0, 0.5 % 416.9 / 403.9, 2 %
+// 416.9 / 418.5, 20 % 417.5 / 420.2; 2048 x 2048, no hole 110.9 / 96.9, 2 %
+// 110.9 / 110.9; 640 x 480 12.4 / 12.3.
+template <int TH, int PPT, int RN>
 __global__ void __launch_bounds__(TILE_W * TH, 4 * 8 / TH)
-    k_initial_normals(const float* __restrict__ depth, int H, int W, Camera cam, int rn, float det_tol,
+    k_initial_normals(const float* __restrict__ depth, int H, int W, Camera cam, int rn_rt, float det_tol,
                       float* __restrict__ normal) {
     extern __shared__ float smem[];
     constexpr int NT = TILE_W * TH;
     constexpr int TROWS = TH * PPT;
+    const int rn = RN > 0 ? RN : rn_rt;
     const int SW = TILE_W + 2 * rn, SH = TROWS + 2 * rn;
     float* tz = smem;
-    // holes[sy] != 0: the staged row sy has a point without a range
+    // RN > 0: holes[sy] != 0: the staged row sy has a point without a range
     int* holes = (int*)(smem + SW * SH);
     const int ub = blockIdx.x * TILE_W, vb = blockIdx.y * TROWS;
     const int tid = threadIdx.y * TILE_W + threadIdx.x;
     // element i = sy SW + sx, advanced by NT per step without a division
     const int dy = NT / SW, dx = NT - dy * SW;
-    for (int i = tid; i < SH; i += NT) holes[i] = 0;
-    __syncthreads();
+    if (RN > 0) {
+        for (int i = tid; i < SH; i += NT) holes[i] = 0;
+        __syncthreads();
+    }
     int sy = tid / SW, sx = tid - sy * SW;
     for (int i = tid; i < SW * SH; i += NT) {
         const int gv = vb - rn + sy, gu = ub - rn + sx;
@@ -124,7 +135,7 @@ __global__ void __launch_bounds__(TILE_W * TH, 4 * 8 / TH)
             if (range_ok(d)) z = d;
         }
         tz[i] = z;
-        if (z == 0.f) holes[sy] = 1;  // every writer stores the same value
+        if (RN > 0 && z == 0.f) holes[sy] = 1;  // every writer stores the same value
         sx += dx;
         sy += dy;
         if (sx >= SW) {
@@ -133,6 +144,16 @@ __global__ void __launch_bounds__(TILE_W * TH, 4 * 8 / TH)
         }
     }
     __syncthreads();
+    // bit k: the patch rows of the warp's k-th pixel row have no hole (lane k looks)
+    unsigned whole = 0;
+    if (RN > 0) {
+        int hole = threadIdx.x >= PPT;
+        if (!hole) {
+#pragma unroll
+            for (int j = 0; j <= 2 * RN; j++) hole |= holes[threadIdx.y + threadIdx.x * TH + j];
+        }
+        whole = __ballot_sync(0xffffffffu, !hole);
+    }
     const int u0 = ub + threadIdx.x;
     if (u0 >= W) return;
 #pragma unroll 1
@@ -144,23 +165,12 @@ __global__ void __launch_bounds__(TILE_W * TH, 4 * 8 / TH)
         const float Zp = tz[cidx];
         float nx = 0.f, ny = 0.f, nz = 1.f;
         bool ok = Zp > 0.f;
-        // the warp's 2 rn + 1 patch rows without a hole: the unmasked sums
-        int hole = rn != NORMAL_RADIUS_UNROLLED;
-        if (rn == NORMAL_RADIUS_UNROLLED) {
-#pragma unroll
-            for (int j = 0; j <= 2 * NORMAL_RADIUS_UNROLLED; j++) hole |= holes[row + j];
-        }
-        if (!hole)
-            ok = initial_normal<NORMAL_RADIUS_UNROLLED, true, true>(tz + cidx, SW, 0, (float)u0 - cam.cx,
-                                                                    (float)v0 - cam.cy, Zp, cam, det_tol, nx, ny,
-                                                                    nz);
+        if (RN > 0 && (whole >> k & 1u))
+            ok = initial_normal<RN, true, true>(tz + cidx, SW, 0, (float)u0 - cam.cx, (float)v0 - cam.cy, Zp, cam,
+                                                det_tol, nx, ny, nz);
         else if (ok)
-            ok = rn == NORMAL_RADIUS_UNROLLED
-                     ? initial_normal<NORMAL_RADIUS_UNROLLED, true>(tz + cidx, SW, 0, (float)u0 - cam.cx,
-                                                                    (float)v0 - cam.cy, Zp, cam, det_tol, nx, ny,
-                                                                    nz)
-                     : initial_normal<0>(tz + cidx, SW, rn, (float)u0 - cam.cx, (float)v0 - cam.cy, Zp, cam,
-                                         det_tol, nx, ny, nz);
+            ok = initial_normal<RN, (RN > 0)>(tz + cidx, SW, rn, (float)u0 - cam.cx, (float)v0 - cam.cy, Zp, cam,
+                                              det_tol, nx, ny, nz);
         const size_t out = (size_t)v0 * W + u0;
         const float q = __int_as_float(0x7fffffff);
         normal[3 * out] = ok ? nx : q;
@@ -196,7 +206,8 @@ cudaError_t launch_backproject(const float* depth, int H, int W, const Camera& c
 // takes the largest PPT that still gives at least two waves of CTAs (a 640 x
 // 480 frame keeps one pixel per thread).
 static size_t initial_normals_smem_bytes(int rn, int ppt) {
-    return (size_t)(TILE_W + 2 * rn + 1) * (NORMAL_TH * ppt + 2 * rn) * sizeof(float);  // Z plane, row flags
+    const int flags = rn == NORMAL_RADIUS_UNROLLED;  // one a staged row
+    return (size_t)(TILE_W + 2 * rn + flags) * (NORMAL_TH * ppt + 2 * rn) * sizeof(float);
 }
 
 template <int PPT>
@@ -205,8 +216,12 @@ static cudaError_t launch_normals_ppt(const float* depth, int H, int W, const Ca
     constexpr int rows = NORMAL_TH * PPT;
     const dim3 block(TILE_W, NORMAL_TH);
     const dim3 grid((W + TILE_W - 1) / TILE_W, (H + rows - 1) / rows);
-    k_initial_normals<NORMAL_TH, PPT>
-        <<<grid, block, initial_normals_smem_bytes(rn, PPT), stream>>>(depth, H, W, cam, rn, det_tol, normal);
+    const size_t smem = initial_normals_smem_bytes(rn, PPT);
+    if (rn == NORMAL_RADIUS_UNROLLED)
+        k_initial_normals<NORMAL_TH, PPT, NORMAL_RADIUS_UNROLLED>
+            <<<grid, block, smem, stream>>>(depth, H, W, cam, rn, det_tol, normal);
+    else
+        k_initial_normals<NORMAL_TH, PPT, 0><<<grid, block, smem, stream>>>(depth, H, W, cam, rn, det_tol, normal);
     return cudaGetLastError();
 }
 

@@ -43,10 +43,10 @@ struct BatchScratch {
     pcurv::BatchTable* h_table[2] = {nullptr, nullptr};  // page-locked host
     cudaEvent_t done[2] = {nullptr, nullptr};
     bool pending[2] = {false, false};
-    // one graph per staging copy and tile variant: batches of changing size
-    // change between 32 x 8 and 32 x 4 tiles, and capturing anew on each change
-    // took 33 us of host time a call instead of 12
-    cudaGraphExec_t graph[2][pcurv::NUM_TILE_VARIANTS] = {};
+    // one graph per staging copy, tile variant and presence of strips: batches of
+    // changing size change between 32 x 8 and 32 x 4 tiles, and capturing anew on
+    // each change took 38 us of host time a call instead of 12
+    cudaGraphExec_t graph[2][pcurv::NUM_TILE_VARIANTS][2] = {};
     cudaStream_t capture = nullptr;           // private stream used only for capture
     int grid[pcurv::NUM_TILE_VARIANTS] = {};  // persistent CTAs per tile variant
     const pcurv::KernelOps* packed_ops = nullptr;  // kernels packed_grid was sized for
@@ -219,10 +219,11 @@ void release_batch(BatchScratch& b) {
     for (int i = 0; i < 2; i++) {
         if (b.pending[i]) cudaEventSynchronize(b.done[i]);
         b.pending[i] = false;
-        for (int v = 0; v < pcurv::NUM_TILE_VARIANTS; v++) {
-            if (b.graph[i][v]) cudaGraphExecDestroy(b.graph[i][v]);
-            b.graph[i][v] = nullptr;
-        }
+        for (auto& variant : b.graph[i])
+            for (cudaGraphExec_t& exec : variant) {
+                if (exec) cudaGraphExecDestroy(exec);
+                exec = nullptr;
+            }
         if (b.h_table[i]) cudaFreeHost(b.h_table[i]);
         b.h_table[i] = nullptr;
         if (b.done[i]) cudaEventDestroy(b.done[i]);
@@ -769,24 +770,25 @@ static pc_status ensure_batch(pc_ctx* ctx, BatchScratch& b, int n) {
 }
 
 // Copy of the staged table, queue reset and persistent kernel (tile variant v,
-// `grid` CTAs), on `s`.
-static cudaError_t enqueue_batch(pc_ctx* ctx, BatchScratch& b, int slot, size_t bytes, int v, int grid,
+// `grid` CTAs, with or without strips), on `s`.
+static cudaError_t enqueue_batch(pc_ctx* ctx, BatchScratch& b, int slot, size_t bytes, int v, int grid, bool strips,
                                  cudaStream_t s) {
     cudaError_t e = cudaMemcpyAsync(b.d_table, b.h_table[slot], bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(b.d_counter, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
-    return pcurv::select_ops(ctx->cfg)->batch[v](b.d_table, b.d_counter, grid, ctx->cfg, s);
+    return pcurv::select_ops(ctx->cfg)->batch[v](b.d_table, b.d_counter, grid, ctx->cfg, strips, s);
 }
 
-// The graph of staging copy `slot` and tile variant v (captured on the private
-// stream once per capacity; release_batch ends it with the buffers it names).
-static pc_status ensure_graph(pc_ctx* ctx, BatchScratch& b, int slot, int v) {
-    cudaGraphExec_t& exec = b.graph[slot][v];
+// The graph of staging copy `slot`, tile variant v and strips (captured on the
+// private stream once per capacity; release_batch ends it with the buffers it
+// names).
+static pc_status ensure_graph(pc_ctx* ctx, BatchScratch& b, int slot, int v, bool strips) {
+    cudaGraphExec_t& exec = b.graph[slot][v][strips];
     if (exec) return PC_OK;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b.capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture begin");
-    const cudaError_t e1 = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(b.cap), v, b.grid[v], b.capture);
+    const cudaError_t e1 = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(b.cap), v, b.grid[v], strips, b.capture);
     e = cudaStreamEndCapture(b.capture, &g);
     if (e1 != cudaSuccess || e != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -843,6 +845,7 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
     }
     pcurv::BatchTable* t = b.h_table[slot];
     int k = 0, begin = 0;
+    bool strips = false;
     for (int i = 0; i < n; i++) {
         const pc_frame& fr = frames[i];
         if (fr.H == 0 || fr.W == 0) continue;
@@ -850,8 +853,10 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
         d.f = pcurv::FrameArgs{fr.depth, fr.H, fr.W,
                                pcurv::Camera{fr.fx, fr.fy, fr.cx, fr.cy, 1.f / fr.fx, 1.f / fr.fy},
                                fr.k1, fr.k2, fr.normal, nullptr, nullptr, 0};
+        const pcurv::Tiling tl = pcurv::tiling_of_variant(fr.H, fr.W, v);
+        strips |= pcurv::has_strips(tl);
         d.tile_begin = begin;
-        begin += (int)pcurv::tiles_of(fr.H, fr.W, v);
+        begin += tl.full + tl.n16 + tl.n8;
     }
     t->nframes = live;
     t->total_tiles = begin;
@@ -863,9 +868,9 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
     // launches bypass the graph, which holds the full grid.
     const int grid = begin < b.grid[v] ? begin : b.grid[v];
     if (ctx->params.batch_graph && grid == b.grid[v]) {
-        if ((st = ensure_graph(ctx, b, slot, v)) != PC_OK) return st;
-        if ((e = cudaGraphLaunch(b.graph[slot][v], s)) != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
-    } else if ((e = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(live), v, grid, s)) != cudaSuccess) {
+        if ((st = ensure_graph(ctx, b, slot, v, strips)) != PC_OK) return st;
+        if ((e = cudaGraphLaunch(b.graph[slot][v][strips], s)) != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
+    } else if ((e = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(live), v, grid, strips, s)) != cudaSuccess) {
         return cuda_fail(ctx, e, "batch launch");
     }
     if ((e = cudaEventRecord(b.done[slot], s)) != cudaSuccess) return cuda_fail(ctx, e, "batch event");
@@ -931,6 +936,7 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
     }
     pcurv::BatchTable* t = b.h_table[slot];
     int k = 0, begin = 0;
+    bool strips = false;
     for (int i = 0; i < n; i++) {
         const pc_packed_frame& fr = frames[i];
         if (fr.H == 0 || fr.W == 0) continue;
@@ -938,8 +944,10 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
         d.f = pcurv::FrameArgs{nullptr, fr.H, fr.W,
                                pcurv::Camera{fr.fx, fr.fy, fr.cx, fr.cy, 1.f / fr.fx, 1.f / fr.fy},
                                fr.k1, fr.k2, fr.normal, fr.packed, fr.tile_base, format};
+        const pcurv::Tiling tl = pcurv::tiling_of_variant(fr.H, fr.W, 0);
+        strips |= pcurv::has_strips(tl);
         d.tile_begin = begin;
-        begin += (int)pcurv::tiles_of(fr.H, fr.W, 0);
+        begin += tl.full + tl.n16 + tl.n8;
     }
     t->nframes = live;
     t->total_tiles = begin;
@@ -948,7 +956,7 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
     if ((e = cudaMemcpyAsync(b.d_table, t, pcurv::batch_table_bytes(live), cudaMemcpyHostToDevice, s)) !=
             cudaSuccess ||
         (e = cudaMemsetAsync(b.d_counter, 0, sizeof(unsigned), s)) != cudaSuccess ||
-        (e = ops->batch[0](b.d_table, b.d_counter, begin < slots ? begin : slots, ctx->cfg, s)) != cudaSuccess)
+        (e = ops->batch[0](b.d_table, b.d_counter, begin < slots ? begin : slots, ctx->cfg, strips, s)) != cudaSuccess)
         return cuda_fail(ctx, e, "packed batch launch");
     if ((e = cudaEventRecord(b.done[slot], s)) != cudaSuccess) return cuda_fail(ctx, e, "batch event");
     b.pending[slot] = true;

@@ -1112,16 +1112,18 @@ __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH
     }
 }
 
-// Dynamic shared memory of a kernel variant: planes, counts and, for the
-// one-thread FP32 kernels, the folded totals of its 32 x TH threads.
+// Dynamic shared memory of a launch of a kernel variant, with or without strip
+// tiles: planes, counts and, for the one-thread FP32 kernels, the folded totals
+// of its 32 x TH threads.
 template <int PREC, int TH, int G>
-size_t variant_smem_bytes(const FitConfig& cfg) {
+size_t variant_smem_bytes(const FitConfig& cfg, bool strips) {
     constexpr bool FOLD = G == 1 && (PREC & PREC_KAHAN) == 0;
-    return fit_smem_bytes(cfg, TH, G == 1, FOLD ? TILE_W * TH : 0);
+    return fit_smem_bytes(cfg, TH, G == 1 && strips, FOLD ? TILE_W * TH : 0);
 }
 
-// Kernels whose dynamic shared memory exceeds the default 48 KB opt in on the
-// current device (idempotent; needed before a launch or occupancy query).
+// Kernels whose dynamic shared memory may exceed the default 48 KB opt in on the
+// current device, for the largest launch under cfg (idempotent; needed before a
+// launch or occupancy query).
 template <typename K>
 cudaError_t allow_smem(K kernel, size_t smem) {
     if (smem <= 48 * 1024) return cudaSuccess;
@@ -1135,11 +1137,10 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
     const int row0 = ty0 * TH, row1 = ty1 * TH < f.H ? ty1 * TH : f.H;
     const Tiling tl = tiling_of(row1 - row0, f.W, TH, G == 1);
     const dim3 strips(tl.full + tl.n16 + tl.n8), columns(tl.cols, (row1 - row0 + TH - 1) / TH);
-    const size_t smem = variant_smem_bytes<PREC, TH, G>(cfg);
     auto launch = [&](auto* kernel, dim3 grid) {
-        const cudaError_t e = allow_smem(kernel, smem);
+        const cudaError_t e = allow_smem(kernel, variant_smem_bytes<PREC, TH, G>(cfg, true));
         if (e != cudaSuccess) return e;
-        kernel<<<grid, block, smem, stream>>>(f, cfg, row0, row1);
+        kernel<<<grid, block, variant_smem_bytes<PREC, TH, G>(cfg, has_strips(tl)), stream>>>(f, cfg, row0, row1);
         return cudaGetLastError();
     };
     // A frame of at most one 128-thread CTA per SM (one warp per scheduler) takes
@@ -1177,16 +1178,16 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
 }
 
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>
-cudaError_t launch_batch_rw(const BatchTable* table, unsigned* next_tile, int grid, const FitConfig& cfg,
+cudaError_t launch_batch_rw(const BatchTable* table, unsigned* next_tile, int grid, const FitConfig& cfg, bool strips,
                             cudaStream_t stream) {
     const dim3 block(TILE_W, TH * G);
-    const size_t smem = variant_smem_bytes<PREC, TH, G>(cfg);
+    const size_t most = variant_smem_bytes<PREC, TH, G>(cfg, true), smem = variant_smem_bytes<PREC, TH, G>(cfg, strips);
     cudaError_t e;
     if (cfg.reject) {
-        if ((e = allow_smem(k_fit_batch<RW, true, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
+        if ((e = allow_smem(k_fit_batch<RW, true, PREC, TH, G, RS>, most)) != cudaSuccess) return e;
         k_fit_batch<RW, true, PREC, TH, G, RS><<<grid, block, smem, stream>>>(table, next_tile, cfg);
     } else {
-        if ((e = allow_smem(k_fit_batch<RW, false, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
+        if ((e = allow_smem(k_fit_batch<RW, false, PREC, TH, G, RS>, most)) != cudaSuccess) return e;
         k_fit_batch<RW, false, PREC, TH, G, RS><<<grid, block, smem, stream>>>(table, next_tile, cfg);
     }
     return cudaGetLastError();
@@ -1194,7 +1195,7 @@ cudaError_t launch_batch_rw(const BatchTable* table, unsigned* next_tile, int gr
 
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>
 cudaError_t occupancy_rw(const FitConfig& cfg, int* blocks_per_sm) {
-    const size_t smem = variant_smem_bytes<PREC, TH, G>(cfg);
+    const size_t smem = variant_smem_bytes<PREC, TH, G>(cfg, true);
     cudaError_t e;
     if (cfg.reject) {
         if ((e = allow_smem(k_fit_batch<RW, true, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;

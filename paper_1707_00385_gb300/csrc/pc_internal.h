@@ -109,10 +109,14 @@ PC_HD inline TilePos tile_pos(const Tiling& t, int i, int th) {
     if (i < t.n16) return TilePos{t.cols * TILE_W, i * 2 * th, 4};
     return TilePos{t.cols * TILE_W + (t.n16 > 0 ? 16 : 0), (i - t.n16) * 4 * th, 3};
 }
+inline Tiling tiling_of_variant(int rows, int W, int variant) {
+    return tiling_of(rows, W, tile_h_of(variant), lanes_of(variant) == 1);
+}
 inline long long tiles_of(int rows, int W, int variant) {
-    const Tiling t = tiling_of(rows, W, tile_h_of(variant), lanes_of(variant) == 1);
+    const Tiling t = tiling_of_variant(rows, W, variant);
     return (long long)t.full + t.n16 + t.n8;
 }
+inline bool has_strips(const Tiling& t) { return t.n16 + t.n8 > 0; }
 
 // First row of the frame that a band ending at row vend does not read.  A strip
 // tile is taller than a tile row and may overhang the band; the band's windows
@@ -129,9 +133,12 @@ PC_HD inline int tile_pitch(int tw, int halo) {
     return tw == 16 ? sw + (48 - sw % 32) % 32 : tw == 8 ? sw + (24 - sw % 16) % 16 : sw;
 }
 
-// Z and c planes of the tile + halo, per-row valid counts (the largest of the
-// tile shapes the variant uses) and, for fold_threads > 0, the folded totals
-// of that many threads (8-byte aligned).
+// Z and c planes of the tile + halo, per-row valid counts (of a 32-pixel tile
+// or, with strips, the largest of the three shapes) and, for fold_threads > 0,
+// the folded totals of that many threads (8-byte aligned).  A launch without a
+// strip asks for what 32-pixel tiles need: what a strip needs more is taken from
+// the L1 cache, which holds the registers a window loop spills (GB300, the 37 x
+// 37 patch with rejection, 64 x 48: 65.7 us, with the strips' request 70.8).
 inline size_t fit_smem_bytes(const FitConfig& c, int th, bool strips, int fold_threads = 0) {
     const int h = halo_of(c);
     size_t planes = 0;
@@ -182,7 +189,9 @@ inline size_t batch_table_bytes(int nframes) {
 struct KernelOps {
     // tile rows [ty0, ty1) of one frame (the variant's tile height)
     cudaError_t (*fit[NUM_TILE_VARIANTS])(const FrameArgs&, const FitConfig&, cudaStream_t, int ty0, int ty1);
-    cudaError_t (*batch[NUM_TILE_VARIANTS])(const BatchTable*, unsigned*, int, const FitConfig&, cudaStream_t);
+    // the persistent kernel over a table of tiles, with or without strips among them
+    cudaError_t (*batch[NUM_TILE_VARIANTS])(const BatchTable*, unsigned*, int grid, const FitConfig&, bool strips,
+                                            cudaStream_t);
     cudaError_t (*occupancy[NUM_TILE_VARIANTS])(const FitConfig&, int*);
 };
 

@@ -139,6 +139,7 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
 
     pcurv::BatchTable* t = (pcurv::BatchTable*)g_host_table;
     int k = 0, begin = 0;
+    bool strips = false;
     for (int i = 0; i < n; i++) {
         const pc_frame& f = frames[i];
         if (f.H == 0 || f.W == 0) continue;
@@ -146,8 +147,10 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
         d.f = pcurv::FrameArgs{f.depth, f.H, f.W,
                                pcurv::Camera{f.fx, f.fy, f.cx, f.cy, 1.f / f.fx, 1.f / f.fy},
                                f.k1, f.k2, f.normal, nullptr, nullptr, 0};
+        const pcurv::Tiling tl = pcurv::tiling_of_variant(f.H, f.W, v);
+        strips |= pcurv::has_strips(tl);
         d.tile_begin = begin;
-        begin += (int)pcurv::tiles_of(f.H, f.W, v);
+        begin += tl.full + tl.n16 + tl.n8;
     }
     t->nframes = live;
     t->total_tiles = begin;
@@ -164,7 +167,7 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
     if ((e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s)) != cudaSuccess)
         return fail(ctx, PC_ERR_CUDA, "counter reset", e);
     // one CTA per tile when the queue is shorter than the persistent grid
-    if ((e = ops->batch[v](table, counter, begin < slots ? begin : slots, cfg, s)) != cudaSuccess)
+    if ((e = ops->batch[v](table, counter, begin < slots ? begin : slots, cfg, strips, s)) != cudaSuccess)
         return fail(ctx, PC_ERR_CUDA, "launch", e);
     return PC_OK;
 }

@@ -80,7 +80,9 @@ int main() {
             if (pitch < tw + 2 * halo || banks != 0xffffffffu) { printf("pitch %d of %d, halo %d\n", pitch, tw, halo); return 1; }
             for (int th : {8, 4}) {
                 const size_t rows = 32 * th / tw + 2 * halo, need = pitch * rows * 8 + rows * tw * 4;
-                if (fit_smem_bytes(c, th, true) < need) { printf("planes of %d, halo %d\n", tw, halo); return 1; }
+                if (fit_smem_bytes(c, th, tw < 32) < need) { printf("planes of %d, halo %d\n", tw, halo); return 1; }
+                // without strips no more than the 32-pixel tile, rounded up to 8 bytes
+                if (tw == 32 && fit_smem_bytes(c, th, false) >= need + 8) { printf("halo %d: too much\n", halo); return 1; }
             }
         }
     }

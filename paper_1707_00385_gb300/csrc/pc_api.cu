@@ -356,11 +356,17 @@ bool plan_allows(const pc_ctx* ctx, int v) { return ctx->params.lanes_per_pixel 
 // smaller windows).  The smaller tiles are taken where they end first: r = 7,
 // 352 x 264 (363 or 726 tiles) 222.7 against 193.7 us, 512 x 384 435 against
 // 408, 160 x 120 81 against 57, while 192 x 144 stays at 80.6 against 86.7 and
-// r = 4, T = 2 at 835 x 507 stays at 144 against 168.
+// r = 4, T = 2 at 835 x 507 stays at 144 against 168.  With rejection and an
+// unrolled radius of 8 and more, a pixel itself takes longer in a CTA of 128
+// threads (measured at 640 x 480 and 1280 x 720, beyond the staging: 1.5 and 4 %
+// at r = 8, 5 and 8, 8 and 11, 13, 12 at r = 12): 682 x 579, r = 11 2796 us with
+// 32 x 8 tiles, 3088 with 32 x 4 ones, which end a step earlier.
 int heuristic_variant(const pcurv::FitConfig& c, long long tiles8, long long tiles4, int sms) {
     const long long steps8 = (tiles8 + sms - 1) / sms, steps4 = (tiles4 + sms - 1) / sms;
     const long long side = 2 * (c.r / c.stride) + 1, work = c.T * (side * side + 25) + 60;
-    return steps4 * (work + 60) < 2 * steps8 * work ? 1 : 0;
+    static const int reject_percent[] = {1, 6, 8, 13, 12};  // radius 8 to 12
+    const long long extra = c.reject && c.stride == 1 && c.r >= 8 && c.r <= 12 ? work * reject_percent[c.r - 8] / 100 : 0;
+    return steps4 * (work + 60 + extra) < 2 * steps8 * work ? 1 : 0;
 }
 
 // Tile variant for one H x W image: forced, tuned, or the heuristic (one lane

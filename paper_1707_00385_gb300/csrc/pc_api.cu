@@ -610,8 +610,10 @@ pc_status pc_compute_packed(pc_ctx* ctx, const unsigned short* packed, const flo
         !is_device_ptr(k1_out) || !is_device_ptr(k2_out) || (normal_out && !is_device_ptr(normal_out)))
         return PC_ERR_INVALID_ARG;
     const pcurv::FrameArgs f{nullptr, H, W, ctx->cam, k1_out, k2_out, normal_out, packed, tile_base, format};
-    const cudaError_t e =
-        fit_frame(pcurv::select_packed_ops(ctx->cfg), 0, f, ctx->cfg, (cudaStream_t)stream);
+    int sms = 0;
+    cudaError_t e = sm_count(ctx, &sms);  // the launch goes by it (FitConfig::sms)
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "pc_compute_packed");
+    e = fit_frame(pcurv::select_packed_ops(ctx->cfg), 0, f, ctx->cfg, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "pc_compute_packed launch");
     return PC_OK;
 }

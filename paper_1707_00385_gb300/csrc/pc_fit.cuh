@@ -47,6 +47,7 @@
 //     then meets a sum over a few rows instead of the whole window.
 #pragma once
 #include <cfloat>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include <cuda_bf16.h>
@@ -945,8 +946,10 @@ __device__ __forceinline__ void fit_tile(const FrameArgs& f, const FitConfig& cf
         // The window's row addresses are the same in every iteration.  Made opaque
         // here, they are computed again instead of all being kept in registers,
         // which spilled for small windows (GB300, 640 x 480, T = 5, a frame
-        // batched: r = 2 94.3 -> 88.4 us, r = 14 2.404 -> 2.314 ms alone).
-        if (STRIPS) asm volatile("" : "+r"(SW));
+        // batched: r = 2 94.3 -> 88.4 us, r = 14 2.404 -> 2.314 ms alone).  Radius 1
+        // with rejection, whose few addresses fit, is 10 % slower with it (61.5
+        // against 55.4 us).
+        if (STRIPS && !(RW == 1 && REJECT)) asm volatile("" : "+r"(SW));
         const float *zc = tz + cidx, *cc = tcv + cidx;
         Moments2 m, comp;
         zero(m);
@@ -1136,13 +1139,23 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
     const dim3 block(TILE_W, TH * G);
     const int row0 = ty0 * TH, row1 = ty1 * TH < f.H ? ty1 * TH : f.H;
     const Tiling tl = tiling_of(row1 - row0, f.W, TH, G == 1);
-    const dim3 strips(tl.full + tl.n16 + tl.n8), columns(tl.cols, (row1 - row0 + TH - 1) / TH);
-    auto launch = [&](auto* kernel, dim3 grid) {
+    const dim3 strips(tl.full + tl.n16 + tl.n8);
+    auto launch = [&](auto* kernel, dim3 grid, bool has_strip_tiles) {
         const cudaError_t e = allow_smem(kernel, variant_smem_bytes<PREC, TH, G>(cfg, true));
         if (e != cudaSuccess) return e;
-        kernel<<<grid, block, variant_smem_bytes<PREC, TH, G>(cfg, has_strips(tl)), stream>>>(f, cfg, row0, row1);
+        kernel<<<grid, block, variant_smem_bytes<PREC, TH, G>(cfg, has_strip_tiles), stream>>>(f, cfg, row0, row1);
         return cudaGetLastError();
     };
+    // a form with and without rejection, in the grid it takes
+    auto launch_form = [&](auto form) {
+        constexpr Form FORM = decltype(form)::value;
+        const bool strip_tiles = FORM != COLUMNS && has_strips(tl);
+        const dim3 grid = FORM == COLUMNS ? dim3((f.W + TILE_W - 1) / TILE_W, (row1 - row0 + TH - 1) / TH) : strips;
+        return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, FORM>, grid, strip_tiles)
+                          : launch(k_fit<RW, false, PREC, TH, G, RS, FORM>, grid, strip_tiles);
+    };
+    using InColumns = std::integral_constant<Form, COLUMNS>;
+    using WithStrips = std::integral_constant<Form, STRIPS>;
     // A frame of at most one 128-thread CTA per SM (one warp per scheduler) takes
     // the roomy form, which the SM could hold two of.  GB300, 160 x 120 / 109 x
     // 82, T = 5, against 128 registers: r = 3 15.2 -> 14.3 / 15.9 -> 14.4 us, r =
@@ -1151,30 +1164,37 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
     // level with it (0.96 to 1.05), and two CTAs per SM are no faster than one
     // 32 x 8 tile.
     if constexpr (PREC == 0 && G == 1 && TH == 4 && (RW / RS >= 5 || RW / RS == 3)) {
-        if (!cfg.reject && (int)strips.x <= cfg.sms) return launch(k_fit<RW, false, PREC, TH, G, RS, ROOMY>, strips);
+        if (!cfg.reject && (int)strips.x <= cfg.sms)
+            return launch(k_fit<RW, false, PREC, TH, G, RS, ROOMY>, strips, has_strips(tl));
     }
     // Plain sums over windows of 5 to 7 samples' radius keep, where there are no
     // strips, the form that knows the tile's shape when compiled, whose loop needs
     // no more registers than it has (GB300, 640 x 480 frames alone: r = 6 3.577
     // against 3.640 ms for eight, the 37 x 37 patch 3.622 against 3.690, r = 7
     // 4.621 against 4.638); elsewhere the form with strips is as fast or faster.
-    if constexpr ((PREC & ~PREC_PACKED) == 0 && G == 1 && RW / RS >= 5 && RW / RS <= 7) {
-        if (tl.n16 + tl.n8 == 0)
-            return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, COLUMNS>, columns)
-                              : launch(k_fit<RW, false, PREC, TH, G, RS, COLUMNS>, columns);
+    // At 6 samples that form costs 2 to 5 % (323 x 241, 32 x 4 tiles: r = 6 149.8
+    // against 153.9 us, the 37 x 37 patch 152.7 against 159.9), at radius 1 up to 6
+    // (323 x 241 with rejection 22.7 against 24.2), with compensated sums up to 4
+    // (323 x 241, r = 1 47.3 against 49.3; with rejection it is the faster one, 257
+    // against 265 at 160 x 120, r = 7 from FP16 storage): there, strips that save
+    // the SM with the most tiles none of them are left out too.
+    constexpr bool KAHAN = (PREC & PREC_KAHAN) != 0;
+    if constexpr (G == 1 && (KAHAN || RW == 1 || (RW / RS >= 5 && RW / RS <= 7))) {
+        const Tiling whole = tiling_of(row1 - row0, f.W, TH, false);
+        auto steps = [&](int tiles) { return (tiles + cfg.sms - 1) / cfg.sms; };
+        const bool idle = (KAHAN || RW == 1 || RW / RS == 6) && cfg.sms > 0 && steps((int)strips.x) == steps(whole.full);
+        if (!(KAHAN && cfg.reject) && (!has_strips(tl) || idle)) return launch_form(InColumns{});
     }
     // So do the run-time loops with rejection in frames of few tiles, ragged or
     // not (64 x 49, T = 5: r = 14 328 us against 356 with the general form, r = 12
-    // sampled every 3 41.5 against 45.2; from 320 x 241 up the two are level).
-    if constexpr (PREC == 0 && G == 1 && RW == 0) {
-        const Tiling tc = tiling_of(row1 - row0, f.W, TH, false);
-        if (cfg.reject && (tl.n16 + tl.n8 == 0 || tc.full <= 2 * cfg.sms))
-            return launch(k_fit<RW, true, PREC, TH, G, RS, COLUMNS>, dim3(tc.cols, (row1 - row0 + TH - 1) / TH));
+    // sampled every 3 41.5 against 45.2, from FP16 storage 160 x 120 473 against
+    // 491 and 107 against 111; from 320 x 241 up the two are level).
+    if constexpr (!KAHAN && G == 1 && RW == 0) {
+        const Tiling whole = tiling_of(row1 - row0, f.W, TH, false);
+        if (cfg.reject && (!has_strips(tl) || whole.full <= 2 * cfg.sms)) return launch_form(InColumns{});
     }
-    constexpr Form FORM = G == 1 ? STRIPS : COLUMNS;
-    const dim3 grid = G == 1 ? strips : columns;
-    return cfg.reject ? launch(k_fit<RW, true, PREC, TH, G, RS, FORM>, grid)
-                      : launch(k_fit<RW, false, PREC, TH, G, RS, FORM>, grid);
+    if constexpr (G > 1) return launch_form(InColumns{});
+    else return launch_form(WithStrips{});
 }
 
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>

@@ -53,3 +53,23 @@ def test_same_bits_as_a_width_without_strips(gpu, rem, H, th, r, kw):
         assert np.array_equal(a, b, equal_nan=True)
         assert np.array_equal(a, o.cpu().numpy(), equal_nan=True)
         assert np.array_equal(a, h.numpy(), equal_nan=True)
+
+
+# the windows that leave strips out where those save no step of an SM (33 rows), and take them where they do (2000)
+@pytest.mark.parametrize("H", [33, 2000])
+@pytest.mark.parametrize("rem", [3, 20])
+@pytest.mark.parametrize("r,kw", [(1, {}), (1, {"reject": 1}), (6, {}), (18, {"stride": 3}), (5, {"kahan": 1}),
+                                  (5, {"kahan": 1, "reject": 1})])
+def test_strips_left_out_or_taken(gpu, rem, H, r, kw):
+    import torch
+    W = 32 + rem
+    z = surface(H, W)
+    c = gpu.Curvature(525.0, 525.0, 20.0, H / 2.0, window_radius=r, iterations=3, **kw)
+    d = torch.from_numpy(z).cuda()
+    wide = np.zeros((H, 64), np.float32)
+    wide[:, :W] = z
+    got = [t.cpu().numpy() for t in c(d)]
+    want = [t.cpu().numpy()[:, :W] for t in c(torch.from_numpy(wide).cuda())]
+    c.close()
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b, equal_nan=True)

@@ -43,10 +43,10 @@ struct BatchScratch {
     pcurv::BatchTable* h_table[2] = {nullptr, nullptr};  // page-locked host
     cudaEvent_t done[2] = {nullptr, nullptr};
     bool pending[2] = {false, false};
-    // one graph per staging copy, tile variant and presence of strips: batches of
+    // one graph per staging copy, tile variant and form of the kernel: batches of
     // changing size change between 32 x 8 and 32 x 4 tiles, and capturing anew on
     // each change took 38 us of host time a call instead of 12
-    cudaGraphExec_t graph[2][pcurv::NUM_TILE_VARIANTS][2] = {};
+    cudaGraphExec_t graph[2][pcurv::NUM_TILE_VARIANTS][pcurv::NUM_BATCH_FORMS] = {};
     cudaStream_t capture = nullptr;           // private stream used only for capture
     int grid[pcurv::NUM_TILE_VARIANTS] = {};  // persistent CTAs per tile variant
     const pcurv::KernelOps* packed_ops = nullptr;  // kernels packed_grid was sized for
@@ -778,25 +778,25 @@ static pc_status ensure_batch(pc_ctx* ctx, BatchScratch& b, int n) {
 }
 
 // Copy of the staged table, queue reset and persistent kernel (tile variant v,
-// `grid` CTAs, with or without strips), on `s`.
-static cudaError_t enqueue_batch(pc_ctx* ctx, BatchScratch& b, int slot, size_t bytes, int v, int grid, bool strips,
-                                 cudaStream_t s) {
+// `grid` CTAs), on `s`.
+static cudaError_t enqueue_batch(pc_ctx* ctx, BatchScratch& b, int slot, size_t bytes, int v, int grid,
+                                 pcurv::BatchForm form, cudaStream_t s) {
     cudaError_t e = cudaMemcpyAsync(b.d_table, b.h_table[slot], bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(b.d_counter, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
-    return pcurv::select_ops(ctx->cfg)->batch[v](b.d_table, b.d_counter, grid, ctx->cfg, strips, s);
+    return pcurv::select_ops(ctx->cfg)->batch[v](b.d_table, b.d_counter, grid, ctx->cfg, form, s);
 }
 
-// The graph of staging copy `slot`, tile variant v and strips (captured on the
+// The graph of staging copy `slot`, tile variant v and form (captured on the
 // private stream once per capacity; release_batch ends it with the buffers it
 // names).
-static pc_status ensure_graph(pc_ctx* ctx, BatchScratch& b, int slot, int v, bool strips) {
-    cudaGraphExec_t& exec = b.graph[slot][v][strips];
+static pc_status ensure_graph(pc_ctx* ctx, BatchScratch& b, int slot, int v, pcurv::BatchForm form) {
+    cudaGraphExec_t& exec = b.graph[slot][v][form];
     if (exec) return PC_OK;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b.capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture begin");
-    const cudaError_t e1 = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(b.cap), v, b.grid[v], strips, b.capture);
+    const cudaError_t e1 = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(b.cap), v, b.grid[v], form, b.capture);
     e = cudaStreamEndCapture(b.capture, &g);
     if (e1 != cudaSuccess || e != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -875,10 +875,11 @@ static pc_status batch_on(pc_ctx* ctx, BatchScratch& b, const pc_frame* frames, 
     // tiles, 150 tiles on a 608-CTA grid, took 88 us against 58 us).  Such
     // launches bypass the graph, which holds the full grid.
     const int grid = begin < b.grid[v] ? begin : b.grid[v];
+    const pcurv::BatchForm form = pcurv::batch_form(strips, begin, b.grid[v]);
     if (ctx->params.batch_graph && grid == b.grid[v]) {
-        if ((st = ensure_graph(ctx, b, slot, v, strips)) != PC_OK) return st;
-        if ((e = cudaGraphLaunch(b.graph[slot][v][strips], s)) != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
-    } else if ((e = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(live), v, grid, strips, s)) != cudaSuccess) {
+        if ((st = ensure_graph(ctx, b, slot, v, form)) != PC_OK) return st;
+        if ((e = cudaGraphLaunch(b.graph[slot][v][form], s)) != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
+    } else if ((e = enqueue_batch(ctx, b, slot, pcurv::batch_table_bytes(live), v, grid, form, s)) != cudaSuccess) {
         return cuda_fail(ctx, e, "batch launch");
     }
     if ((e = cudaEventRecord(b.done[slot], s)) != cudaSuccess) return cuda_fail(ctx, e, "batch event");
@@ -964,7 +965,7 @@ pc_status pc_compute_packed_batch(pc_ctx* ctx, const pc_packed_frame* frames, in
     if ((e = cudaMemcpyAsync(b.d_table, t, pcurv::batch_table_bytes(live), cudaMemcpyHostToDevice, s)) !=
             cudaSuccess ||
         (e = cudaMemsetAsync(b.d_counter, 0, sizeof(unsigned), s)) != cudaSuccess ||
-        (e = ops->batch[0](b.d_table, b.d_counter, begin < slots ? begin : slots, ctx->cfg, strips, s)) != cudaSuccess)
+        (e = ops->batch[0](b.d_table, b.d_counter, begin < slots ? begin : slots, ctx->cfg, pcurv::batch_form(strips, begin, slots), s)) != cudaSuccess)
         return cuda_fail(ctx, e, "packed batch launch");
     if ((e = cudaEventRecord(b.done[slot], s)) != cudaSuccess) return cuda_fail(ctx, e, "batch event");
     b.pending[slot] = true;

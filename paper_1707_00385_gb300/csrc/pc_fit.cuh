@@ -47,6 +47,7 @@
 //     then meets a sum over a few rows instead of the whole window.
 #pragma once
 #include <cfloat>
+#include <climits>
 #include <type_traits>
 #include <cuda_runtime.h>
 
@@ -1090,7 +1091,9 @@ __global__ void __launch_bounds__(TILE_W * TH * G, FORM == ROOMY ? 8 / TH : PC_B
 // still gets one item per SM -- then items gridDim.x, gridDim.x + 1, ... with
 // one atomic each.  The header and descriptors live in device memory
 // (BatchTable); *next_tile must be 0 at launch.
-template <int RW, bool REJECT, int PREC, int TH, int G, int RS>
+// FEW: the form for a short queue without strips (batch_form): 32-pixel columns
+// only, no state formed a pair ahead.
+template <int RW, bool REJECT, int PREC, int TH, int G, int RS, bool FEW>
 __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH * G)))
     k_fit_batch(const BatchTable* __restrict__ table, unsigned* __restrict__ next_tile, FitConfig cfg) {
     extern __shared__ float smem[];
@@ -1105,14 +1108,30 @@ __global__ void __launch_bounds__(TILE_W * TH * G, PC_BLOCKS_OF(PREC) * (8 / (TH
             const int mid = (lo + hi + 1) >> 1;
             if (fr[mid].tile_begin <= t) lo = mid; else hi = mid - 1;
         }
-        const int H = fr[lo].f.H;
-        const TilePos p = tile_pos(tiling_of(H, fr[lo].f.W, TH, G == 1), t - fr[lo].tile_begin, TH);
-        fit_tile<RW, REJECT, PREC, TH, G, RS, G == 1, PC_AHEAD_BATCH>(fr[lo].f, cfg, p.ub, p.vb, p.lg, H, smem);
+        const int H = fr[lo].f.H, local = t - fr[lo].tile_begin;
+        if constexpr (FEW) {
+            const int cols = (fr[lo].f.W + TILE_W - 1) / TILE_W, row = local / cols;
+            fit_tile<RW, REJECT, PREC, TH, G, RS, false, INT_MAX>(fr[lo].f, cfg, (local - row * cols) * TILE_W, row * TH, 5,
+                                                                  H, smem);
+        } else {
+            const TilePos p = tile_pos(tiling_of(H, fr[lo].f.W, TH, G == 1), local, TH);
+            fit_tile<RW, REJECT, PREC, TH, G, RS, G == 1, PC_AHEAD_BATCH>(fr[lo].f, cfg, p.ub, p.vb, p.lg, H, smem);
+        }
         __syncthreads();  // shared memory and s_tile are reused by the next tile
         if (threadIdx.x == 0 && threadIdx.y == 0) s_tile = (int)(gridDim.x + atomicAdd(next_tile, 1u));
         __syncthreads();
         t = s_tile;
     }
+}
+
+// The windows whose short queues have a kernel of their own (k_fit_batch, FEW):
+// those for which it is faster.  The run-time loops with rejection are faster
+// with strips' registers also there (512 x 424, r = 12 sampled every 2: 552 us
+// against 644), and radius 1 to 5 level.
+__host__ __device__ constexpr bool few_form(int rw, int rs, int prec, int g, bool reject) {
+    if (g != 1 || (prec & PREC_KAHAN)) return false;
+    if (rw == 0) return !reject;
+    return rw / rs >= 6 && (!reject || (prec == 0 && rw >= 11));
 }
 
 // Dynamic shared memory of a launch of a kernel variant, with or without strip
@@ -1198,19 +1217,24 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
 }
 
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>
-cudaError_t launch_batch_rw(const BatchTable* table, unsigned* next_tile, int grid, const FitConfig& cfg, bool strips,
+cudaError_t launch_batch_rw(const BatchTable* table, unsigned* next_tile, int grid, const FitConfig& cfg, BatchForm form,
                             cudaStream_t stream) {
     const dim3 block(TILE_W, TH * G);
-    const size_t most = variant_smem_bytes<PREC, TH, G>(cfg, true), smem = variant_smem_bytes<PREC, TH, G>(cfg, strips);
-    cudaError_t e;
-    if (cfg.reject) {
-        if ((e = allow_smem(k_fit_batch<RW, true, PREC, TH, G, RS>, most)) != cudaSuccess) return e;
-        k_fit_batch<RW, true, PREC, TH, G, RS><<<grid, block, smem, stream>>>(table, next_tile, cfg);
-    } else {
-        if ((e = allow_smem(k_fit_batch<RW, false, PREC, TH, G, RS>, most)) != cudaSuccess) return e;
-        k_fit_batch<RW, false, PREC, TH, G, RS><<<grid, block, smem, stream>>>(table, next_tile, cfg);
+    auto launch = [&](auto* kernel) {
+        const cudaError_t e = allow_smem(kernel, variant_smem_bytes<PREC, TH, G>(cfg, true));
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, block, variant_smem_bytes<PREC, TH, G>(cfg, form == BATCH_STRIPS), stream>>>(table, next_tile, cfg);
+        return cudaGetLastError();
+    };
+    // the kernel for short queues, where it is faster (FEW_TILES)
+    if constexpr (few_form(RW, RS, PREC, G, false)) {
+        if (form == BATCH_FEW && !cfg.reject) return launch(k_fit_batch<RW, false, PREC, TH, G, RS, true>);
     }
-    return cudaGetLastError();
+    if constexpr (few_form(RW, RS, PREC, G, true)) {
+        if (form == BATCH_FEW && cfg.reject) return launch(k_fit_batch<RW, true, PREC, TH, G, RS, true>);
+    }
+    return cfg.reject ? launch(k_fit_batch<RW, true, PREC, TH, G, RS, false>)
+                      : launch(k_fit_batch<RW, false, PREC, TH, G, RS, false>);
 }
 
 template <int RW, int PREC, int TH, int G = 1, int RS = 1>
@@ -1218,12 +1242,12 @@ cudaError_t occupancy_rw(const FitConfig& cfg, int* blocks_per_sm) {
     const size_t smem = variant_smem_bytes<PREC, TH, G>(cfg, true);
     cudaError_t e;
     if (cfg.reject) {
-        if ((e = allow_smem(k_fit_batch<RW, true, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_fit_batch<RW, true, PREC, TH, G, RS>,
+        if ((e = allow_smem(k_fit_batch<RW, true, PREC, TH, G, RS, false>, smem)) != cudaSuccess) return e;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_fit_batch<RW, true, PREC, TH, G, RS, false>,
                                                              TILE_W * TH * G, smem);
     }
-    if ((e = allow_smem(k_fit_batch<RW, false, PREC, TH, G, RS>, smem)) != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_fit_batch<RW, false, PREC, TH, G, RS>,
+    if ((e = allow_smem(k_fit_batch<RW, false, PREC, TH, G, RS, false>, smem)) != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_fit_batch<RW, false, PREC, TH, G, RS, false>,
                                                          TILE_W * TH * G, smem);
 }
 

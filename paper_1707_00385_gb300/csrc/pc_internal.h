@@ -172,6 +172,23 @@ struct BatchFrame {
     int pad;
 };
 
+// Forms of the persistent kernel over a table of tiles: with strips among them,
+// with 32-pixel columns only, and with columns only in a queue so short that its
+// end counts (k_fit_batch).
+enum BatchForm { BATCH_STRIPS, BATCH_COLUMNS, BATCH_FEW, NUM_BATCH_FORMS };
+// Tiles per CTA of the persistent grid up to which a queue is short.  The state
+// formed a pair ahead and the registers of the strips pay in a queue of many
+// tiles; where the last tiles of the SMs decide, or a warp is alone on its
+// scheduler, they cost more than they give.  GB300, T = 5, without / with a kernel
+// for short queues: one 640 x 480 frame r = 9 1035 / 940 us, r = 10 1220 / 1137,
+// two of r = 7 1239 / 1189, three of r = 7 level (12 tiles a CTA); one 64 x 48
+// frame r = 12 150 / 141, the 37 x 37 patch 56.8 / 52.7, with rejection 512 x 424
+// 574 / 510.
+constexpr int FEW_TILES = 8;
+inline BatchForm batch_form(bool strips, int tiles, int grid) {
+    return strips ? BATCH_STRIPS : tiles / FEW_TILES < grid ? BATCH_FEW : BATCH_COLUMNS;
+}
+
 // Device-resident batch table: header followed by nframes descriptors.
 struct BatchTable {
     int nframes;
@@ -189,8 +206,7 @@ inline size_t batch_table_bytes(int nframes) {
 struct KernelOps {
     // tile rows [ty0, ty1) of one frame (the variant's tile height)
     cudaError_t (*fit[NUM_TILE_VARIANTS])(const FrameArgs&, const FitConfig&, cudaStream_t, int ty0, int ty1);
-    // the persistent kernel over a table of tiles, with or without strips among them
-    cudaError_t (*batch[NUM_TILE_VARIANTS])(const BatchTable*, unsigned*, int grid, const FitConfig&, bool strips,
+    cudaError_t (*batch[NUM_TILE_VARIANTS])(const BatchTable*, unsigned*, int grid, const FitConfig&, BatchForm,
                                             cudaStream_t);
     cudaError_t (*occupancy[NUM_TILE_VARIANTS])(const FitConfig&, int*);
 };

@@ -167,7 +167,7 @@ extern "C" pc_status pc_compute_batch_static(pc_ctx* ctx, const pc_frame* frames
     if ((e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s)) != cudaSuccess)
         return fail(ctx, PC_ERR_CUDA, "counter reset", e);
     // one CTA per tile when the queue is shorter than the persistent grid
-    if ((e = ops->batch[v](table, counter, begin < slots ? begin : slots, cfg, strips, s)) != cudaSuccess)
+    if ((e = ops->batch[v](table, counter, begin < slots ? begin : slots, cfg, pcurv::batch_form(strips, begin, slots), s)) != cudaSuccess)
         return fail(ctx, PC_ERR_CUDA, "launch", e);
     return PC_OK;
 }

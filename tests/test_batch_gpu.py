@@ -223,6 +223,20 @@ def test_largest_batch(gpu):
     c.close()
 
 
+# queues of one tile, of about one and eight tiles per CTA of the persistent grid and more, without strips and with
+@pytest.mark.parametrize("n,H,W", [(1, 4, 32), (1, 48, 64), (2, 480, 640), (3, 480, 640), (2, 241, 323)])
+@pytest.mark.parametrize("r,kw", [(6, {}), (9, {}), (12, {"reject": 1}), (18, {"stride": 3}), (18, {"stride": 3, "reject": 1}),
+                                  (14, {}), (9, {"tile_height": 4})])
+def test_short_and_long_queues_equal_per_frame(gpu, n, H, W, r, kw):
+    s = synth.kinect_scene(31)
+    scenes = [synth.kinect_scene(31 + i, H=H, W=W) if H >= 200 else synth.crop(s, 100 + i, 120, H, W) for i in range(n)]
+    c = gpu.Curvature(525.0, 525.0, 0.0, 0.0, window_radius=r, iterations=2, **kw)
+    for want, got in zip(per_frame(gpu, scenes, r, 2, **kw), batched(gpu, c, scenes)):
+        for a, b in zip(want, got):
+            assert same(a, b)
+    c.close()
+
+
 def test_alternating_tile_heights_do_not_capture_anew(gpu):
     """Two batches that take different tile heights, in turn: the results of
     each alone, and a call takes no more than twice the host time it takes when

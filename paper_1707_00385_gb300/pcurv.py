@@ -260,39 +260,32 @@ def _frame_array(frames):
     The descriptors are written with one struct call each (0.135 ms for 256
     frames on the GB300's host; through ctypes constructors such a batch of 64 x
     48 frames took 455 us a call, bound by the host, now 261, bound by the
-    kernel), which a value out of a C type's range refuses; ctypes then converts
-    it, and the library checks it."""
+    kernel).  struct refuses a value out of a C type's range: ctypes converts
+    that frame, and the library checks it."""
     buf = bytearray(_FRAME.size * len(frames))
-    try:
-        for i, (d, (fx, fy, cx, cy), a, b, n) in enumerate(frames):
-            H, W = d.shape
-            _FRAME.pack_into(buf, i * _FRAME.size, d.data_ptr(), H, W, fx, fy, cx, cy, a.data_ptr(), b.data_ptr(),
-                             0 if n is None else n.data_ptr())
-    except (OverflowError, struct.error):
-        arr = (pc_frame * len(frames))()
-        for i, (d, intr, a, b, n) in enumerate(frames):
-            H, W = d.shape
-            arr[i] = pc_frame(d.data_ptr(), H, W, *map(float, intr), a.data_ptr(), b.data_ptr(),
-                              n.data_ptr() if n is not None else None)
-        return arr
+    for i, (d, (fx, fy, cx, cy), a, b, n) in enumerate(frames):
+        H, W = d.shape
+        k1, k2, normal = a.data_ptr(), b.data_ptr(), 0 if n is None else n.data_ptr()
+        try:
+            _FRAME.pack_into(buf, i * _FRAME.size, d.data_ptr(), H, W, fx, fy, cx, cy, k1, k2, normal)
+        except (OverflowError, struct.error):
+            buf[i * _FRAME.size:(i + 1) * _FRAME.size] = bytes(
+                pc_frame(d.data_ptr(), H, W, *map(float, (fx, fy, cx, cy)), k1, k2, normal))
     return (pc_frame * len(frames)).from_buffer(buf)
 
 
 def _packed_frame_array(frames):
     """The same of pc_packed_frame for (packed, tile_base, intrinsics, k1, k2, normal) tuples."""
     buf = bytearray(_PACKED_FRAME.size * len(frames))
-    try:
-        for i, (q, base, (fx, fy, cx, cy), a, b, n) in enumerate(frames):
-            H, W = q.shape
-            _PACKED_FRAME.pack_into(buf, i * _PACKED_FRAME.size, q.data_ptr(), base.data_ptr(), H, W, fx, fy, cx, cy,
-                                    a.data_ptr(), b.data_ptr(), 0 if n is None else n.data_ptr())
-    except (OverflowError, struct.error):
-        arr = (pc_packed_frame * len(frames))()
-        for i, (q, base, intr, a, b, n) in enumerate(frames):
-            H, W = q.shape
-            arr[i] = pc_packed_frame(q.data_ptr(), base.data_ptr(), H, W, *map(float, intr), a.data_ptr(),
-                                     b.data_ptr(), n.data_ptr() if n is not None else None)
-        return arr
+    for i, (q, base, (fx, fy, cx, cy), a, b, n) in enumerate(frames):
+        H, W = q.shape
+        k1, k2, normal = a.data_ptr(), b.data_ptr(), 0 if n is None else n.data_ptr()
+        try:
+            _PACKED_FRAME.pack_into(buf, i * _PACKED_FRAME.size, q.data_ptr(), base.data_ptr(), H, W, fx, fy, cx, cy, k1,
+                                    k2, normal)
+        except (OverflowError, struct.error):
+            buf[i * _PACKED_FRAME.size:(i + 1) * _PACKED_FRAME.size] = bytes(
+                pc_packed_frame(q.data_ptr(), base.data_ptr(), H, W, *map(float, (fx, fy, cx, cy)), k1, k2, normal))
     return (pc_packed_frame * len(frames)).from_buffer(buf)
 
 

@@ -250,8 +250,9 @@ def _stream_handle(stream):
     if stream is not None:
         return stream.cuda_stream
     import torch
-    # torch.cuda.current_stream() without building its Stream object
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    # torch.cuda.current_stream() without building its Stream object, where torch has it
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
 
 
 def _frame_array(frames):

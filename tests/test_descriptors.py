@@ -46,3 +46,15 @@ def test_bytes_of_the_structures(once):
         assert len(got) == len(ref)
         for g, w in zip(got, ref):
             assert bytes(g) == bytes(w)
+
+
+def test_stream_of_a_torch_without_the_raw_handle(monkeypatch):
+    torch = pytest.importorskip("torch")
+
+    class Stream:
+        cuda_stream = 17
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert pcurv._stream_handle(None) == 17
+    assert pcurv._stream_handle(Stream) == 17

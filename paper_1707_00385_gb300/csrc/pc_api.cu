@@ -12,6 +12,7 @@
 
 #include "../../include/pcurv.h"
 #include "pc_internal.h"
+#include "pc_pointers.h"
 
 // The fused kernels stage halo rows of at most 96 columns (three warp ballots).
 static_assert(pcurv::TILE_W + 2 * PC_MAX_RADIUS <= 96 && PC_MAX_NORMAL_RADIUS <= PC_MAX_RADIUS,
@@ -128,27 +129,13 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// The device pointers of one call.  A pointer inside an allocation that holds
-// another pointer of the call needs no query of its own: a batch of frames cut
-// from a few allocations asks the driver a few times instead of four times a
-// frame.  An allocation counts when its last byte is a device pointer too.
-// Nothing is kept from one call for the next.
-class DevicePtrs {
-  public:
-    bool operator()(const void* p) {
-        const uintptr_t a = (uintptr_t)p;
-        for (int i = 0; i < used_; i++)
-            if (a >= lo_[i] && a < hi_[i]) return true;
-        if (!is_device_ptr(p)) return false;
-        CUdeviceptr base = 0;
-        size_t size = 0;
-        const AddressRange range = address_range();
-        if (range && range(&base, &size, (CUdeviceptr)a) == CUDA_SUCCESS && size > 0 && a >= base && a - base < size &&
-            is_device_ptr((const void*)(base + size - 1))) {
-            const int i = used_ < MAX ? used_++ : next_++ % MAX;
-            lo_[i] = base;
-            hi_[i] = base + size;
-        }
+struct DriverPointers {
+    static bool is_device(const void* p) { return is_device_ptr(p); }
+    static bool range(const void* p, uintptr_t* base, size_t* size) {
+        const AddressRange f = address_range();
+        CUdeviceptr b = 0;
+        if (!f || f(&b, size, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return false;
+        *base = (uintptr_t)b;
         return true;
     }
 
@@ -168,10 +155,8 @@ class DevicePtrs {
         }();
         return f;
     }
-    static constexpr int MAX = 8;
-    uintptr_t lo_[MAX], hi_[MAX];
-    int used_ = 0, next_ = 0;
 };
+using DevicePtrs = pcurv::DevicePointers<DriverPointers>;
 
 pc_status check_params(const pc_params& p) {
     if (!(finite_f(p.k) && p.k > 0.f)) return PC_ERR_INVALID_ARG;

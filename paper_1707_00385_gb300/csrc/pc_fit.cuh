@@ -1181,7 +1181,11 @@ cudaError_t launch_fit_rw(const FrameArgs& f, const FitConfig& cfg, cudaStream_t
     // 7 57.4 -> 49.1 / 57.5 -> 49.4, r = 12 141 -> 116 / 141 -> 115, the 37 x 37
     // patch 1.08 / 1.19 times as fast.  Radii 1 and 4 and the run-time kernels are
     // level with it (0.96 to 1.05), and two CTAs per SM are no faster than one
-    // 32 x 8 tile.
+    // 32 x 8 tile.  The rule looks at one frame: on several streams at once, frames
+    // of 160 x 120 gain on two (r = 7 8 %, r = 3 3) and lose what the smaller
+    // number of resident CTAs costs on eight (r = 7 3 %, r = 3 and the 37 x 37 patch
+    // 7 to 8), while 109 x 82 and 64 x 48 gain on eight, too (4 to 10 %, r = 3 and
+    // the patch 0 to 5); many small frames are faster in one batch.
     if constexpr (PREC == 0 && G == 1 && TH == 4 && (RW / RS >= 5 || RW / RS == 3)) {
         if (!cfg.reject && (int)strips.x <= cfg.sms)
             return launch(k_fit<RW, false, PREC, TH, G, RS, ROOMY>, strips, has_strips(tl));

@@ -1,7 +1,7 @@
-// Instantiations for ranges stored as 16-bit offsets from a per-tile base, with radius and stride read
-// at run time (r = 0) and for dense windows of radius 1 to 6, unrolled
-// (plain sums, 32 x 8 tiles).  The arithmetic after loading a range is the
-// float32 kernels' own.
+// Instantiations for ranges stored as 16-bit offsets from a per-tile base, with
+// radius and stride read at run time (r = 0) and for dense windows of radius 1
+// to 6, unrolled (plain sums, 32 x 8 tiles).  The arithmetic after loading a
+// range is the float32 kernels' own.
 #include "pc_fit.cuh"
 
 namespace pcurv {

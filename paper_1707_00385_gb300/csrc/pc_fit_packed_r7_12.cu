@@ -1,7 +1,6 @@
-// Instantiations for ranges stored as 16-bit offsets from a per-tile base, for dense windows of radius
-// 7 to 12, unrolled
-// (plain sums, 32 x 8 tiles).  The arithmetic after loading a range is the
-// float32 kernels' own.
+// Instantiations for ranges stored as 16-bit offsets from a per-tile base, for
+// dense windows of radius 7 to 12, unrolled (plain sums, 32 x 8 tiles).  The
+// arithmetic after loading a range is the float32 kernels' own.
 #include "pc_fit.cuh"
 
 namespace pcurv {

@@ -76,7 +76,7 @@ def outputs(H, W, device="cuda"):
 
 CONFIGS = [(7, {}), (7, {"tile_height": 4}), (7, {"lanes_per_pixel": 2}), (7, {"lanes_per_pixel": 4}),
            (7, {"lanes_per_pixel": 8}), (1, {}), (12, {}), (15, {}), (7, {"stride": 3}), (5, {"reject": 1}),
-           (18, {"stride": 3}), (3, {"kahan": 1}), (7, {"fp64_solve_cond": 1e6, "pivot_tol": 1e-7})]
+           (18, {"stride": 3}), (3, {"kahan": 1}), (5, {"kahan": 1}), (12, {"kahan": 1}), (7, {"fp64_solve_cond": 1e6, "pivot_tol": 1e-7})]
 
 
 @pytest.mark.parametrize("r,params", CONFIGS, ids=[f"r{r}-" + "-".join(f"{k}{v}" for k, v in p.items())
@@ -162,8 +162,7 @@ def test_packed_storage_stays_in_bounds(gpu, frames, fmt):
 @pytest.mark.parametrize("r", [3, 5, 11])
 @pytest.mark.parametrize("fmt", [1, 2])
 def test_packed_batch_stays_in_bounds(gpu, frames, fmt, r):
-    """pc_compute_packed_batch over every shape at once (unrolled radii 3 and
-    11, run-time radius 5)."""
+    """pc_compute_packed_batch over every shape at once (unrolled radii 3, 5 and 11)."""
     import torch
     c = ctx(gpu, next(iter(frames.values())), r)
     arr = (gpu.pc_packed_frame * len(frames))()

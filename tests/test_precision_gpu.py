@@ -75,8 +75,7 @@ def test_pack_rounds_each_offset_once(gpu, scene, fmt):
 @pytest.mark.parametrize("fmt", [1, 2])
 def test_packed_path_equals_fp32_path_on_decoded_ranges(gpu, scene, fmt, r):
     """The arithmetic after loading is the FP32 path's: same bits on the
-    decoded ranges (3, 7 and 11 have window loops unrolled for the 16-bit
-    loads, 5 takes the general one)."""
+    decoded ranges (all four have window loops unrolled for the 16-bit loads)."""
     import torch
     c = gpu.Curvature(*scene.intrinsics, window_radius=r, iterations=5)
     d = torch.from_numpy(scene.depth).cuda()

@@ -84,7 +84,8 @@ typedef struct pc_params {
     int min_window;      /* fewest valid window points accepted. Default 6 */
     int batch_graph;     /* 1 = pc_compute_batch replays a CUDA graph (copy of the frame table,
                             reset of the tile queue, persistent kernel) captured once per
-                            table capacity; 0 = enqueue the three steps directly.  A batch
+                            table capacity, tile height and form of the kernel (columns only,
+                            strips, short queues); 0 = enqueue the three steps directly.  A batch
                             with fewer tiles than the persistent grid is always enqueued
                             directly, with one CTA per tile. Default 1 */
     int kahan;           /* 1 = compensated (Kahan) summation of the window moments in FP32;
@@ -95,8 +96,8 @@ typedef struct pc_params {
                             pivots. 0 = off (default) */
     int tile_height;     /* pixel rows of the 32-column tile one CTA computes with one thread per
                             pixel: 8 or 4; 0 = choose per image (the size's pc_autotune result
-                            when there is one, else 8 when the image has at least 1.5 32x8
-                            tiles per SM, else 4).  Results do not depend on it.  Default 0 */
+                            when there is one, else the height with which the SM that has the
+                            most tiles ends first).  Results do not depend on it.  Default 0 */
     int lanes_per_pixel; /* threads that share one pixel's window: 2, 4 or 8 lanes of a warp
                             split the window rows and add their moment sums by shuffles before
                             each solve (tiles of 32 x 8/lanes pixels, 256 threads).  For images

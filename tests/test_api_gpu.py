@@ -193,6 +193,40 @@ def test_argument_errors_leave_outputs_untouched(gpu):
     c.close()
 
 
+@pytest.mark.parametrize("packed", [False, True])
+def test_batch_checks_every_pointer(gpu, packed):
+    """Frames from more allocations than a call keeps the range of, the last one
+    with a host pointer (pageable, then page-locked) in each place in turn: the
+    call is refused and nothing is written; with device memory there it runs."""
+    import torch
+    H, W, n = 16, 32, 12
+    c = gpu.Curvature(525.0, 525.0, 16.0, 8.0, 3, 2)
+    frames = []
+    for _ in range(n):
+        # above the size that torch's allocator cuts several tensors from one allocation
+        block = torch.full((24 << 20,), 1.0, dtype=torch.uint8, device="cuda").view(torch.float32)
+        d, k1, k2 = (block[i * 4096:i * 4096 + H * W].view(H, W) for i in range(3))
+        normal = block[4 * 4096:4 * 4096 + 3 * H * W].view(H, W, 3)
+        d.fill_(1.0)
+        for t in (k1, k2, normal):
+            t.fill_(7.0)
+        src = c.pack(d, 1) if packed else (d,)
+        frames.append((*src, (525.0, 525.0, 16.0, 8.0), k1, k2, normal))
+    run = (lambda f: c.batch_packed(f, 1)) if packed else c.batch
+    last = frames[-1]
+    for place in [i for i, t in enumerate(last) if isinstance(t, torch.Tensor)]:
+        for host in (last[place].cpu(), last[place].cpu().pin_memory()):
+            with pytest.raises(gpu.PcError) as e:
+                run(frames[:-1] + [last[:place] + (host,) + last[place + 1:]])
+            assert e.value.status == gpu.PC_ERR_INVALID_ARG
+    torch.cuda.synchronize()
+    assert all(bool((t == 7.0).all()) for f in frames for t in f[-3:])
+    run(frames)
+    torch.cuda.synchronize()
+    assert not any(bool((t == 7.0).any()) for f in frames for t in f[-3:])
+    c.close()
+
+
 def test_contexts_on_concurrent_streams(gpu):
     """Four contexts on four streams, each with per-frame, batch and host-batch
     calls in flight at once, give the bits of the same calls run one after
